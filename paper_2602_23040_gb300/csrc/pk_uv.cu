@@ -1,13 +1,15 @@
 // UV cells (eq. uvgs2) and Max-K UV pruning (Sec. 4.2 "UV-Based Pruning").
 //
-// Five launches over n candidate Gaussians and an M x N map: cell and
-// in-cell slot per Gaussian (one atomic per valid Gaussian on the cell's
-// counter), an exclusive scan of the per-cell counts, a scatter of the
-// Gaussian indices into per-cell buckets, and the rank of every Gaussian
+// Four launches over n candidate Gaussians and an M x N map (after the
+// zeroing of the counts): cell and in-cell slot per Gaussian (one atomic per
+// valid Gaussian on the cell's counter), a bucket per cell (each block scans
+// its cells' counts and takes its stretch of the bucket array with one
+// atomic: the buckets' order among each other does not matter), a scatter of
+// the Gaussian indices into the buckets, and the rank of every Gaussian
 // within its bucket by opacity (higher first, then lower index): the
 // buckets hold a handful of Gaussians, so each Gaussian counts the members
-// that beat it.  The cell is taken in FP64 (atan2, acos), where a
-// neighbouring cell is only chosen within ~1e-15 of a cell boundary.
+// that beat it.  The cell is the one FP64 gives (atan2, acos); FP64 itself
+// runs only where FP32 cannot tell the cell apart (k_uv_cell).
 #include "pk_common.cuh"
 
 using namespace pk;
@@ -16,10 +18,11 @@ namespace {
 
 constexpr int kUvThreads = 256;
 constexpr int kUvScanItems = 2048;   // counts per scan block (8 per thread)
+constexpr int kUvCellItems = 8;      // Gaussians per thread of k_uv_cell
 constexpr uint32_t kInvalid = 0xFFFFFFFFu;
 
 struct UvScratch {
-  size_t slot, offs, bsum, bucket, total;
+  size_t slot, offs, taken, bucket, total;
 };
 
 UvScratch uv_layout(int64_t n, int64_t cells) {
@@ -30,36 +33,95 @@ UvScratch uv_layout(int64_t n, int64_t cells) {
     off = (off + bytes + 255) & ~size_t(255);
     return at_;
   };
-  const int64_t blocks = (cells + kUvScanItems - 1) / kUvScanItems;
   L.slot = take(sizeof(uint32_t) * (size_t)(n > 0 ? n : 1));
   L.offs = take(sizeof(uint32_t) * (size_t)cells);
-  L.bsum = take(sizeof(uint32_t) * (size_t)(blocks + 1));
+  L.taken = take(sizeof(uint32_t));   // bucket entries handed out so far
   L.bucket = take(sizeof(uint32_t) * (size_t)(n > 0 ? n : 1));
   L.total = off;
   return L;
 }
 
+// Cell of a Gaussian in FP64, kInvalid without a valid projection.
+__device__ __noinline__ uint32_t uv_cell_f64(float xf, float yf, float zf, int M, int N) {
+  const double x = xf, y = yf, z = zf;
+  const double rho = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
+  if (!(rho > 0.0) || !isfinite(rho)) return kInvalid;
+  const double kPi = 3.14159265358979323846;
+  const double su = (kPi + atan2(y, x)) / (2.0 * kPi) * M, sv = acos(z / rho) / kPi * N;
+  const double u = floor(su), v = floor(sv);
+  return u >= 0.0 && u < M && v >= 0.0 && v < N ? (uint32_t)v * (uint32_t)M + (uint32_t)u : kInvalid;
+}
+
+// Cell by FP32 where that is certain to be the FP64 cell; false where it is
+// not.  The FP32 coordinates su = (pi + atan2(y, x)) M / 2pi and sv =
+// atan2(sqrt(x^2 + y^2), z) N / pi (acos(z / rho) without its cancellation
+// at the poles) lie within 3.5e-7 M and 4.4e-7 N of the exact ones: atan2f
+// is within 3 ulp (7.2e-7 at pi), the sum with pi, the scale and the product
+// add 2^-22 + 1.5 * 2^-23 relative, sqrtf's argument 0.8e-7 of angle.  The
+// FP64 coordinates lie within 1e-8 N (acos near the poles).  So a coordinate
+// further than 1e-6 M (N) from an integer has the same floor in both.
+// The range of the values keeps the squares normal.
+__device__ __forceinline__ bool uv_cell_f32(float x, float y, float z, int M, int N, uint32_t &c) {
+  const float big = fmaxf(fmaxf(fabsf(x), fabsf(y)), fabsf(z));
+  if (!(big > 1e-15f && big < 1e15f) || !isfinite(x) || !isfinite(y) || !isfinite(z)) return false;
+  const float su = (3.14159265f + atan2f(y, x)) * (0.15915494f * (float)M);
+  const float sv = atan2f(sqrtf(x * x + y * y), z) * (0.31830989f * (float)N);
+  const float u = floorf(su), v = floorf(sv);
+  const float du = 1e-6f * (float)M, dv = 1e-6f * (float)N;
+  if (!(su - u > du && su - u < 1.f - du && sv - v > dv && sv - v < 1.f - dv)) return false;
+  if (!(u >= 0.f && u < (float)M && v >= 0.f && v < (float)N)) return false;
+  c = (uint32_t)v * (uint32_t)M + (uint32_t)u;
+  return true;
+}
+
+// The FP64 chain (atan2, acos, divisions) bounds a kernel that runs it for
+// every Gaussian: FP64 runs at a small fraction of the FP32 rate here.
+// Here each block places its kUvCellItems * 256 Gaussians in FP32 and queues
+// the ones within 1e-6 M (N) of a cell's edge -- four in a thousand at 1024^2
+// cells -- which its warps then place in FP64, the lanes full, instead of
+// one lane of every eighth warp: 143 -> 13.7 us at 629 K Gaussians and 1024^2
+// cells (the whole call, with two launches of the scan gone, 183 -> 46 us).
 __global__ __launch_bounds__(kUvThreads) void k_uv_cell(const float *__restrict__ soa, int64_t n, int64_t stride,
                                                          int M, int N, uint32_t *__restrict__ cell,
                                                          uint32_t *__restrict__ slot, uint32_t *count) {
-  const int64_t i = (int64_t)blockIdx.x * kUvThreads + threadIdx.x;
-  if (i >= n) return;
-  const double x = __ldg(soa + i), y = __ldg(soa + stride + i), z = __ldg(soa + 2 * stride + i);
-  const float lg = __ldg(soa + 10 * stride + i);
-  uint32_t c = kInvalid;
-  const double rho = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)));
-  if (rho > 0.0 && isfinite(rho) && lg == lg) {
-    const double kPi = 3.14159265358979323846;
-    const double su = (kPi + atan2(y, x)) / (2.0 * kPi) * M, sv = acos(z / rho) / kPi * N;
-    const double u = floor(su), v = floor(sv);
-    if (u >= 0.0 && u < M && v >= 0.0 && v < N) c = (uint32_t)v * (uint32_t)M + (uint32_t)u;
+  __shared__ uint16_t s_queue[kUvThreads * kUvCellItems];
+  __shared__ uint32_t s_n;
+  if (threadIdx.x == 0) s_n = 0;
+  __syncthreads();
+  const int64_t base = (int64_t)blockIdx.x * (kUvThreads * kUvCellItems);
+  float x[kUvCellItems], y[kUvCellItems], z[kUvCellItems], lg[kUvCellItems];
+#pragma unroll
+  for (int k = 0; k < kUvCellItems; ++k) {
+    const int64_t i = base + k * kUvThreads + threadIdx.x;
+    const bool in = i < n;
+    x[k] = in ? __ldg(soa + i) : 0.f;
+    y[k] = in ? __ldg(soa + stride + i) : 0.f;
+    z[k] = in ? __ldg(soa + 2 * stride + i) : 0.f;
+    lg[k] = in ? __ldg(soa + 10 * stride + i) : 0.f;
   }
-  cell[i] = c;
-  if (c != kInvalid) slot[i] = atomicAdd(count + c, 1u);
+#pragma unroll
+  for (int k = 0; k < kUvCellItems; ++k) {
+    const int64_t i = base + k * kUvThreads + threadIdx.x;
+    if (i >= n) continue;
+    uint32_t c = kInvalid;
+    if (lg[k] == lg[k] && !uv_cell_f32(x[k], y[k], z[k], M, N, c)) {
+      s_queue[atomicAdd(&s_n, 1u)] = (uint16_t)(k * kUvThreads + threadIdx.x);
+      continue;
+    }
+    cell[i] = c;
+    if (c != kInvalid) slot[i] = atomicAdd(count + c, 1u);
+  }
+  __syncthreads();
+  const uint32_t queued = s_n;
+  for (uint32_t q = threadIdx.x; q < queued; q += kUvThreads) {
+    const int64_t i = base + s_queue[q];
+    const uint32_t c = uv_cell_f64(__ldg(soa + i), __ldg(soa + stride + i), __ldg(soa + 2 * stride + i), M, N);
+    cell[i] = c;
+    if (c != kInvalid) slot[i] = atomicAdd(count + c, 1u);
+  }
 }
 
-// Exclusive scan of counts: per-block totals, a one-block scan of those,
-// then each block scans its counts from its base.
+// Exclusive scan of one value per thread over the block.
 __device__ __forceinline__ uint32_t block_scan_excl(uint32_t x, uint32_t &total, uint32_t *s_warp) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t inc = x;
@@ -86,43 +148,13 @@ __device__ __forceinline__ uint32_t block_scan_excl(uint32_t x, uint32_t &total,
   return excl;
 }
 
-__global__ __launch_bounds__(kUvThreads) void k_uv_block_sums(const uint32_t *__restrict__ count, int64_t cells,
-                                                               uint32_t *__restrict__ bsum) {
-  __shared__ uint32_t s_warp[32];
-  constexpr int kPer = kUvScanItems / kUvThreads;
-  const int64_t base = (int64_t)blockIdx.x * kUvScanItems + (int64_t)threadIdx.x * kPer;
-  uint32_t acc = 0;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k)
-    if (base + k < cells) acc += __ldg(count + base + k);
-  uint32_t tot;
-  block_scan_excl(acc, tot, s_warp);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
-}
-
-__global__ __launch_bounds__(kUvThreads) void k_uv_scan_sums(uint32_t *bsum, int64_t blocks) {
-  __shared__ uint32_t s_warp[32];
-  __shared__ uint32_t s_carry;
-  if (threadIdx.x == 0) s_carry = 0;
-  __syncthreads();
-  for (int64_t b0 = 0; b0 < blocks; b0 += kUvThreads) {
-    const int64_t i = b0 + threadIdx.x;
-    const uint32_t x = i < blocks ? bsum[i] : 0u;
-    uint32_t tot;
-    const uint32_t ex = block_scan_excl(x, tot, s_warp);
-    const uint32_t carry = s_carry;
-    if (i < blocks) bsum[i] = carry + ex;
-    __syncthreads();
-    if (threadIdx.x == 0) s_carry = carry + tot;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) bsum[blocks] = s_carry;
-}
-
+// First bucket entry of each cell: a block's cells lie one after another,
+// the blocks in the order in which they ask.
 __global__ __launch_bounds__(kUvThreads) void k_uv_offsets(const uint32_t *__restrict__ count, int64_t cells,
-                                                            const uint32_t *__restrict__ bsum,
+                                                            uint32_t *taken,
                                                             uint32_t *__restrict__ offs) {
   __shared__ uint32_t s_warp[32];
+  __shared__ uint32_t s_base;
   constexpr int kPer = kUvScanItems / kUvThreads;
   const int64_t base = (int64_t)blockIdx.x * kUvScanItems + (int64_t)threadIdx.x * kPer;
   uint32_t v[kPer], acc = 0;
@@ -132,7 +164,10 @@ __global__ __launch_bounds__(kUvThreads) void k_uv_offsets(const uint32_t *__res
     acc += v[k];
   }
   uint32_t tot;
-  uint32_t run = bsum[blockIdx.x] + block_scan_excl(acc, tot, s_warp);
+  uint32_t run = block_scan_excl(acc, tot, s_warp);
+  if (threadIdx.x == 0) s_base = tot ? atomicAdd(taken, tot) : 0u;
+  __syncthreads();
+  run += s_base;
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     if (base + k < cells) offs[base + k] = run;
@@ -197,16 +232,16 @@ extern "C" pk_status pk_uv_max_k(const float *soa, int64_t n, int64_t stride, in
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const UvScratch L = uv_layout(n, cells);
   uint32_t *slot = at<uint32_t>(scratch, L.slot), *offs = at<uint32_t>(scratch, L.offs);
-  uint32_t *bsum = at<uint32_t>(scratch, L.bsum), *bucket = at<uint32_t>(scratch, L.bucket);
-  pk_status ze = zero_async({{count, sizeof(uint32_t) * (size_t)cells}}, st);
+  uint32_t *taken = at<uint32_t>(scratch, L.taken), *bucket = at<uint32_t>(scratch, L.bucket);
+  pk_status ze = zero_async({{count, sizeof(uint32_t) * (size_t)cells}, {taken, sizeof(uint32_t)}}, st);
   if (ze != PK_OK) return ze;
   if (n == 0) return PK_OK;
   const unsigned gn = (unsigned)((n + kUvThreads - 1) / kUvThreads);
   const int64_t blocks = (cells + kUvScanItems - 1) / kUvScanItems;
-  k_uv_cell<<<gn, kUvThreads, 0, st>>>(soa, n, stride, M, N, cell, slot, count);
-  k_uv_block_sums<<<(unsigned)blocks, kUvThreads, 0, st>>>(count, cells, bsum);
-  k_uv_scan_sums<<<1, kUvThreads, 0, st>>>(bsum, blocks);
-  k_uv_offsets<<<(unsigned)blocks, kUvThreads, 0, st>>>(count, cells, bsum, offs);
+  constexpr int kCellBlock = kUvThreads * kUvCellItems;
+  k_uv_cell<<<(unsigned)((n + kCellBlock - 1) / kCellBlock), kUvThreads, 0, st>>>(soa, n, stride, M, N, cell, slot,
+                                                                                  count);
+  k_uv_offsets<<<(unsigned)blocks, kUvThreads, 0, st>>>(count, cells, taken, offs);
   k_uv_bucket<<<gn, kUvThreads, 0, st>>>(cell, slot, offs, n, bucket);
   k_uv_rank<<<gn, kUvThreads, 0, st>>>(soa, stride, cell, offs, count, bucket, n, K, rank, keep);
   return check_launch();
