@@ -3,23 +3,29 @@
 //
 // One CTA per 32 x 32 output tile of one channel of one view.  It stages
 // the 52 x 52 input window of image and target (halo 2 x 5) in shared
-// memory, forms the five window sums (X, Y, XX, YY, XY) on the 42 x 42
+// memory, forms the four window sums (X, Y, XX + YY, XY: the SSIM
+// value needs the variances' sum alone) on the 42 x 42
 // region (halo 5) by a horizontal then a vertical 11-tap pass, turns them
 // into the SSIM value and its partial derivatives, and sums those back onto
 // the 32 x 32 tile with the same separable window (the adjoint of the
 // window sums).  Every pass is register-tiled: a thread produces 4 to 8
 // consecutive outputs of one row or column from one sliding read of the
 // inputs, so shared-memory reads are about 1/4 of the multiply-adds.  The
-// sums travel in pairs -- (X, Y), (XX, YY) and, backwards, (d1, d11) -- so
-// each tap is one packed FP32 multiply-add per pair (two round-to-nearest
-// results, each the scalar one) plus one scalar for the fifth sum.
+// sums travel in pairs -- (X, Y), (XX + YY, XY) and, backwards, (d1, d11)
+// -- so each tap is one packed FP32 multiply-add per pair (two
+// round-to-nearest results, each the scalar one), and backwards one scalar
+// for d12.
 // Image and target are read once per tile (plus halo) and the gradient
 // written once; the arithmetic (about 400 FP32 operations per value)
 // bounds the kernel.  The five barrier-separated stages each leave some
 // threads idle, so the SM is kept busy by CTAs at different stages: the
 // derivative maps reuse the shared memory of the input window (the last
 // stage reads its centre values again from global memory, where they are
-// still cached), which brings a CTA to 67 KB and three CTAs onto an SM.
+// still cached), which brings a CTA to 58 KB and three CTAs onto an SM.
+// Shared-memory wavefronts (about 75 per 32 values), packed multiply-adds
+// and issue slots each take 1.5 to 1.9 ms of the 4.20 ms at the 52-view rig
+// (234 M values); a fifth sum and four reciprocals per value instead of two
+// took 4.72 ms.
 #include "pk_common.cuh"
 #include "pk_f32x2.cuh"
 
@@ -48,17 +54,14 @@ constexpr int kGE = 4;   // stage E: tile rows per item (32 = 8 x 4)
 
 struct SsimSmem {
   union {
-    struct {
-      float x[kI][kIP], y[kI][kIP];   // inputs, 0 outside the image (read by the horizontal sums only)
-    };
+    f32x2 xy[kI][kIP];                // inputs (X, Y), 0 outside the image (read by the horizontal sums only)
     struct {
       f32x2 d01[kM][kMP];             // then: partial derivatives of the SSIM map, (d1, d11) and d12
       float d2[kM][kMP];
     };
   };
-  f32x2 h01[kI][kMP], h23[kI][kMP];   // horizontal sums (X, Y), (XX, YY); later the backward
-  float h4[kI][kMP];                  //   sums ((d1, d11) pairs, d12) on [kM][kTP]; XY
-};
+  f32x2 h01[kI][kMP], h23[kI][kMP];   // horizontal sums (X, Y), (XX + YY, XY); later the backward
+};                                    //   sums (d1, d11) in h01 and d12 in h23, on [kM][kTP]
 static_assert(sizeof(float) * 2 * kM * kMP + sizeof(float) * kM * kMP <= sizeof(float) * 2 * kI * kIP,
               "the derivative maps fit in the input tiles they replace");
 
@@ -107,72 +110,64 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
       const int i = tid + k * kSsimThreads;
       if (i < kI * kI) {
         const int r = i / kI, q = i - r * kI;
-        S.x[r][q] = xv[k];
-        S.y[r][q] = yv[k];
+        S.xy[r][q] = pack2(xv[k], yv[k]);
       }
     }
   }
   __syncthreads();
-  // B: horizontal window sums of X, Y, XX, YY, XY: each item one input row
+  // B: horizontal window sums of X, Y, XX + YY, XY: each item one input row
   // and kGB consecutive window-sum columns (threads walk down the rows)
   for (int it = tid; it < kI * (kM / kGB); it += kSsimThreads) {
     const int g = it / kI, r = it - g * kI, q0 = g * kGB;
     f32x2 a01[kGB], a23[kGB];
-    float a4[kGB];
 #pragma unroll
     for (int o = 0; o < kGB; ++o) {
       a01[o] = z2;
       a23[o] = z2;
-      a4[o] = 0.f;
     }
 #pragma unroll
     for (int t = 0; t < kGB + 2 * kR; ++t) {
-      const float xv = S.x[r][q0 + t], yv = S.y[r][q0 + t];
-      const f32x2 v = pack2(xv, yv);
-      const f32x2 sq = mul2(v, v);
-      const float xy = xv * yv;
+      const f32x2 v = S.xy[r][q0 + t];
+      float xv, yv;
+      unpack2(v, xv, yv);
+      const f32x2 sq = pack2(fmaf(xv, xv, yv * yv), xv * yv);
 #pragma unroll
       for (int o = 0; o < kGB; ++o) {
         const int j = t - o;
         if (j < 0 || j > 2 * kR) continue;
         a01[o] = fma2(wd[j], v, a01[o]);
         a23[o] = fma2(wd[j], sq, a23[o]);
-        a4[o] = fmaf(w[j], xy, a4[o]);
       }
     }
 #pragma unroll
     for (int o = 0; o < kGB; ++o) {
       S.h01[r][q0 + o] = a01[o];
       S.h23[r][q0 + o] = a23[o];
-      S.h4[r][q0 + o] = a4[o];
     }
   }
   __syncthreads();
   // C: vertical window sums on kGC consecutive rows of one column, then the
-  // SSIM value and its partial derivatives with respect to m1 = G*X,
-  // e11 = G*XX, e12 = G*XY (0 outside the image)
+  // SSIM value s = (A1 / B1) (A2 / B2) and its partial derivatives with
+  // respect to m1 = G*X, e11 = G*XX, e12 = G*XY (0 outside the image); s's
+  // factors p = A1 / B1 and q = A2 / B2 leave two reciprocals per value
   float ssim_sum = 0.f;
   for (int it = tid; it < kM * (kM / kGC); it += kSsimThreads) {
     const int g = it / kM, q = it - g * kM, r0 = g * kGC;
     f32x2 a01[kGC], a23[kGC];
-    float a4[kGC];
 #pragma unroll
     for (int o = 0; o < kGC; ++o) {
       a01[o] = z2;
       a23[o] = z2;
-      a4[o] = 0.f;
     }
 #pragma unroll
     for (int t = 0; t < kGC + 2 * kR; ++t) {
       const f32x2 h01 = S.h01[r0 + t][q], h23 = S.h23[r0 + t][q];
-      const float h4 = S.h4[r0 + t][q];
 #pragma unroll
       for (int o = 0; o < kGC; ++o) {
         const int j = t - o;
         if (j < 0 || j > 2 * kR) continue;
         a01[o] = fma2(wd[j], h01, a01[o]);
         a23[o] = fma2(wd[j], h23, a23[o]);
-        a4[o] = fmaf(w[j], h4, a4[o]);
       }
     }
     const int xx = tx0 - kR + q;
@@ -181,19 +176,18 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
       const int r = r0 + o, yy = ty0 - kR + r;
       float d1 = 0.f, d11 = 0.f, d12 = 0.f;
       if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
-        float m1, m2, e11, e22;
+        float m1, m2, ee, e12;
         unpack2(a01[o], m1, m2);
-        unpack2(a23[o], e11, e22);
-        const float e12 = a4[o];
-        const float A1 = 2.f * m1 * m2 + kC1, A2 = 2.f * (e12 - m1 * m2) + kC2;
-        const float B1 = m1 * m1 + m2 * m2 + kC1, B2 = (e11 - m1 * m1) + (e22 - m2 * m2) + kC2;
+        unpack2(a23[o], ee, e12);
+        const float m12 = m1 * m2, mm = fmaf(m1, m1, m2 * m2);
+        const float A1 = fmaf(2.f, m12, kC1), A2 = fmaf(2.f, e12 - m12, kC2);
+        const float B1 = mm + kC1, B2 = (ee - mm) + kC2;
         // approximate reciprocals (2 ulp): far inside the FP32 tolerance of the loss
-        const float iA1 = __fdividef(1.f, A1), iA2 = __fdividef(1.f, A2), iB1 = __fdividef(1.f, B1),
-                    iB2 = __fdividef(1.f, B2);
-        const float s = A1 * A2 * iB1 * iB2;
-        d1 = 2.f * s * (m2 * (iA1 - iA2) + m1 * (iB2 - iB1));
+        const float iB1 = __fdividef(1.f, B1), iB2 = __fdividef(1.f, B2);
+        const float p = A1 * iB1, qf = A2 * iB2, s = p * qf, pB2 = p * iB2;
+        d1 = 2.f * fmaf(m2, fmaf(qf, iB1, -pB2), m1 * (s * (iB2 - iB1)));
         d11 = -s * iB2;
-        d12 = 2.f * s * iA2;
+        d12 = 2.f * pB2;
         if (r >= kR && r < kR + kT && q >= kR && q < kR + kT) ssim_sum += s;
       }
       S.d01[r][q] = pack2(d1, d11);
@@ -204,7 +198,7 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
   // D: backward horizontal sums of the three maps: one row of the 42 region,
   // kGD consecutive tile columns (into the h buffers, as [kM][kTP])
   f32x2(*hb01)[kTP] = reinterpret_cast<f32x2(*)[kTP]>(&S.h01[0][0]);
-  float(*hb2)[kTP] = reinterpret_cast<float(*)[kTP]>(&S.h4[0][0]);
+  float(*hb2)[kTP] = reinterpret_cast<float(*)[kTP]>(&S.h23[0][0]);
   for (int it = tid; it < kM * (kT / kGD); it += kSsimThreads) {
     const int g = it / kM, r = it - g * kM, q0 = g * kGD;
     f32x2 b01[kGD];
