@@ -2,10 +2,9 @@
 // "Low Precision Optimization").  Live texels of the occupancy mask, in
 // row-major order, become the Gaussians 0..N-1 of every frame.
 //
-// Two kernels: a single-block scan of per-word popcounts (the mask is at
-// most a few hundred thousand words), then one thread per group of four
-// texels that reads each channel with one 16-byte (FP32) or 8-byte (FP16)
-// load and writes the live ones to the channel-major SoA.
+// Two kernels: a scan of the per-word popcounts, then one thread per group
+// of four texels that reads each channel with one 16-byte (FP32) or 8-byte
+// (FP16) load and writes the live ones to the channel-major SoA.
 #include <cuda_fp16.h>
 
 #include "pk_common.cuh"
@@ -15,43 +14,48 @@ using namespace pk;
 namespace {
 
 constexpr int kScanThreads = 1024;
+constexpr int kScanMaxBlocks = 64;
 
 // woff[i] = number of live texels in mask words [0, i); woff[nwords] = total.
-// One block: each pass covers kScanThreads * kRun consecutive words, a run
-// of kRun per thread (popcounts summed in the thread, one block-wide scan of
-// the run totals, then the run's prefixes written back), so a 1024^2 mask
-// takes one pass instead of 32 barrier-separated steps.
-constexpr int kRun = 32;
+// Block b scans words [b per, (b + 1) per), per a multiple of 1024 so that
+// at most kScanMaxBlocks blocks are needed.  It first counts the live texels
+// of all words before its own (16-byte loads; they are L2 hits, and at most
+// 64 blocks read them), so no block waits for another: one launch of a few
+// microseconds where one block walking the whole mask took 11 us at 32 K
+// words.
+__device__ __forceinline__ uint32_t block_sum(uint32_t v, uint32_t *s) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v = __reduce_add_sync(0xffffffffu, v);
+  if (lane == 0) s[warp] = v;
+  __syncthreads();
+  v = __reduce_add_sync(0xffffffffu, s[lane]);
+  __syncthreads();
+  return v;
+}
+
 __global__ __launch_bounds__(kScanThreads) void k_word_scan(const uint32_t *__restrict__ occ, int64_t nwords,
-                                                            uint32_t *__restrict__ woff,
+                                                            int64_t per, uint32_t *__restrict__ woff,
                                                             pk_device_status *status, int64_t N) {
   __shared__ uint32_t s_warp[32];
-  __shared__ uint32_t s_carry;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_carry = 0;
-  __syncthreads();
-  for (int64_t base = 0; base < nwords; base += (int64_t)kScanThreads * kRun) {
-    const int64_t w0 = base + (int64_t)tid * kRun;
-    uint32_t c[kRun];
-    uint32_t tot = 0;
-    if (w0 + kRun <= nwords && (reinterpret_cast<uintptr_t>(occ) & 15u) == 0) {
-      // a whole run: 16-byte loads (the run starts on a 128-byte boundary)
-      const uint4 *q = reinterpret_cast<const uint4 *>(occ + w0);
-#pragma unroll
-      for (int k = 0; k < kRun / 4; ++k) {
-        const uint4 v = __ldg(q + k);
-        c[4 * k] = __popc(v.x);
-        c[4 * k + 1] = __popc(v.y);
-        c[4 * k + 2] = __popc(v.z);
-        c[4 * k + 3] = __popc(v.w);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < kRun; ++k) c[k] = w0 + k < nwords ? __popc(__ldg(occ + w0 + k)) : 0u;
+  const int64_t w0 = (int64_t)blockIdx.x * per, w1 = min(nwords, w0 + per);
+  // live texels before this block (w0 is a multiple of 1024)
+  uint32_t before = 0;
+  if ((reinterpret_cast<uintptr_t>(occ) & 15u) == 0) {
+    const uint4 *q = reinterpret_cast<const uint4 *>(occ);
+#pragma unroll 4
+    for (int64_t i = tid; i < w0 / 4; i += kScanThreads) {
+      const uint4 v = __ldg(q + i);
+      before += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
     }
-#pragma unroll
-    for (int k = 0; k < kRun; ++k) tot += c[k];
-    uint32_t x = tot;
+  } else {
+    for (int64_t i = tid; i < w0; i += kScanThreads) before += __popc(__ldg(occ + i));
+  }
+  uint32_t carry = block_sum(before, s_warp);
+  for (int64_t base = w0; base < w1; base += kScanThreads) {
+    const int64_t i = base + tid;
+    const uint32_t c = i < w1 ? __popc(__ldg(occ + i)) : 0u;
+    uint32_t x = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
@@ -59,48 +63,32 @@ __global__ __launch_bounds__(kScanThreads) void k_word_scan(const uint32_t *__re
     }
     if (lane == 31) s_warp[warp] = x;
     __syncthreads();
-    if (warp == 0) {
-      uint32_t w = s_warp[lane];
+    uint32_t w = s_warp[lane];   // every warp scans the 32 warp totals
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      s_warp[lane] = w;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
     }
-    __syncthreads();
-    const uint32_t carry = s_carry;
-    uint32_t run = carry + (warp ? s_warp[warp - 1] : 0u) + x - tot;
-    if (w0 + kRun <= nwords && (reinterpret_cast<uintptr_t>(woff) & 15u) == 0) {
-      // a whole run: 16-byte stores, a quarter of the store instructions
-      uint4 *o4 = reinterpret_cast<uint4 *>(woff + w0);
-#pragma unroll
-      for (int k = 0; k < kRun / 4; ++k) {
-        uint4 v;
-        v.x = run;
-        v.y = v.x + c[4 * k];
-        v.z = v.y + c[4 * k + 1];
-        v.w = v.z + c[4 * k + 2];
-        run = v.w + c[4 * k + 3];
-        o4[k] = v;
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < kRun; ++k) {
-        if (w0 + k < nwords) woff[w0 + k] = run;
-        run += c[k];
-      }
-    }
-    __syncthreads();
-    if (tid == 0) s_carry = carry + s_warp[31];
-    __syncthreads();
+    const uint32_t mine = __shfl_sync(0xffffffffu, w, (warp + 31) & 31), total = __shfl_sync(0xffffffffu, w, 31);
+    if (i < w1) woff[i] = carry + (warp ? mine : 0u) + x - c;
+    carry += total;
+    __syncthreads();   // before the next chunk's warp totals
   }
-  if (tid == 0) {
-    woff[nwords] = s_carry;
-    status->live_seen = s_carry;
+  if (w1 == nwords && tid == 0) {   // the last block: the whole mask's count
+    woff[nwords] = carry;
+    status->live_seen = carry;
     status->nonfinite = 0;   // counted by the gather kernel that follows
-    if ((int64_t)s_carry != N) atomicOr(&status->flags, PK_DEV_LIVE_MISMATCH);
+    if ((int64_t)carry != N) atomicOr(&status->flags, PK_DEV_LIVE_MISMATCH);
   }
+}
+
+void launch_word_scan(const uint32_t *occ, int64_t nwords, uint32_t *woff, pk_device_status *status, int64_t N,
+                      cudaStream_t st) {
+  int64_t per = (nwords + kScanMaxBlocks - 1) / kScanMaxBlocks;
+  per = (per + kScanThreads - 1) / kScanThreads * kScanThreads;
+  if (per < kScanThreads) per = kScanThreads;
+  const unsigned blocks = (unsigned)((nwords + per - 1) / per);
+  k_word_scan<<<blocks ? blocks : 1u, kScanThreads, 0, st>>>(occ, nwords, per, woff, status, N);
 }
 
 template <typename Tex>
@@ -123,10 +111,11 @@ struct Quad<__half> {
 };
 
 // Live bits and Gaussian indices of the (up to) four texels x0 .. x0 + 3
-// of row y; writes their texel ids and dynamic flags.  False if none is live.
+// of row y; with `write`, writes their texel ids and dynamic flags.  False if
+// none is live.
 __device__ __forceinline__ bool quad_live(const uint32_t *__restrict__ occ, const uint32_t *__restrict__ dyn,
                                           const uint32_t *__restrict__ woff, int W, int y, int x0, int64_t N,
-                                          uint32_t *__restrict__ texel, uint8_t *__restrict__ dynflag,
+                                          bool write, uint32_t *__restrict__ texel, uint8_t *__restrict__ dynflag,
                                           bool live[4], int64_t gidx[4]) {
   const int Wp = (W + 31) / 32;
   bool any = false;
@@ -144,8 +133,10 @@ __device__ __forceinline__ bool quad_live(const uint32_t *__restrict__ occ, cons
           live[i] = true;
           gidx[i] = g;
           any = true;
-          texel[g] = (uint32_t)((int64_t)y * W + x);
-          dynflag[g] = dyn ? (uint8_t)((dyn[(int64_t)y * Wp + (x >> 5)] >> (x & 31)) & 1u) : (uint8_t)1;
+          if (write) {
+            texel[g] = (uint32_t)((int64_t)y * W + x);
+            dynflag[g] = dyn ? (uint8_t)((dyn[(int64_t)y * Wp + (x >> 5)] >> (x & 31)) & 1u) : (uint8_t)1;
+          }
         }
       }
     }
@@ -169,7 +160,7 @@ __global__ __launch_bounds__(256) void k_gather(const Tex *__restrict__ atlas, c
     const int y = (int)(qi / Wq), x0 = (int)(qi % Wq) * 4;
     int64_t gidx[4];
     bool live[4];
-    if (!quad_live(occ, dyn, woff, W, y, x0, N, texel, dynflag, live, gidx)) continue;
+    if (!quad_live(occ, dyn, woff, W, y, x0, N, true, texel, dynflag, live, gidx)) continue;
     const int64_t pix = (int64_t)y * W + x0;
     for (int f = 0; f < F; ++f) {
       uint32_t bad = 0;   // bit i: texel i has a non-finite value in some channel of frame f
@@ -220,7 +211,13 @@ __device__ __forceinline__ uint32_t lpo_code(float x, float lo, float delta, flo
   return (uint32_t)u;
 }
 
-template <bool kCodes>
+// One thread per 4 consecutive texels of a row and group of kChannels
+// channels (blockIdx.y = (frame, group)), whose loads are issued together.
+// kVec: the codes of four texels are one 4-byte load per plane.  At the
+// 1024^2 atlas with 59 channels 116 us with a byte load per texel and all
+// channels in one thread, 87 us so.
+constexpr int kChannels = 8;
+template <bool kCodes, bool kVec>
 __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src, const float *__restrict__ lohi,
                                                     const uint32_t *__restrict__ occ,
                                                     const uint32_t *__restrict__ dyn,
@@ -234,37 +231,76 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
     s_delta[c] = __fdiv_rn(__fsub_rn(lohi[2 * c + 1], lohi[2 * c]), L);
   }
   __syncthreads();
-  const int Wq = (W + 3) / 4;
-  const int64_t nq = (int64_t)Wq * H;
-  const int64_t plane = (int64_t)W * H;
-  const int64_t G = (int64_t)F * N;
-  for (int64_t qi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; qi < nq; qi += (int64_t)gridDim.x * blockDim.x) {
-    const int y = (int)(qi / Wq), x0 = (int)(qi % Wq) * 4;
-    int64_t gidx[4];
-    bool live[4];
-    if (!quad_live(occ, dyn, woff, W, y, x0, N, texel, dynflag, live, gidx)) continue;
-    const int64_t pix = (int64_t)y * W + x0;
-    for (int f = 0; f < F; ++f) {
-      for (int c = 0; c < D; ++c) {
-        const float lo = s_lo[c], delta = s_delta[c];
-        float *dst = soa + (int64_t)c * G + (int64_t)f * N;
+  const uint32_t Wq = (uint32_t)(W + 3) / 4, nq = Wq * (uint32_t)H;
+  const int64_t plane = (int64_t)W * H, G = (int64_t)F * N;
+  const int groups = (D + kChannels - 1) / kChannels;
+  for (int fg = blockIdx.y; fg < F * groups; fg += gridDim.y) {
+    const int f = fg / groups, c0 = (fg - f * groups) * kChannels;
+    for (uint32_t qi = blockIdx.x * blockDim.x + threadIdx.x; qi < nq; qi += gridDim.x * blockDim.x) {
+      const int y = (int)(qi / Wq), x0 = (int)(qi - (uint32_t)y * Wq) * 4;
+      int64_t gidx[4];
+      bool live[4];
+      if (!quad_live(occ, dyn, woff, W, y, x0, N, fg == 0, texel, dynflag, live, gidx)) continue;
+      const int64_t pix = (int64_t)y * W + x0;
+      float *dst = soa + (int64_t)f * N;
+      if (kCodes) {
+        const uint8_t *cb = reinterpret_cast<const uint8_t *>(src) + (int64_t)f * (D + 3) * plane + pix;
+        auto four = [&](int64_t at) -> uint32_t {   // the four texels' bytes of a code plane
+          if (kVec) return __ldg(reinterpret_cast<const uint32_t *>(cb + at));
+          uint32_t v = 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (!live[i]) continue;
-          uint32_t q;
-          if (kCodes) {
-            const uint8_t *cb = reinterpret_cast<const uint8_t *>(src) + (int64_t)f * (D + 3) * plane + pix + i;
-            q = c < 3 ? ((uint32_t)__ldg(cb + (2 * c) * plane) << 8) | __ldg(cb + (2 * c + 1) * plane)
-                      : (uint32_t)__ldg(cb + (c + 3) * plane);
-          } else {
-            const float x = __ldg(reinterpret_cast<const float *>(src) + ((int64_t)f * D + c) * plane + pix + i);
-            q = lpo_code(x, lo, delta, c < 3 ? 65535.0f : 255.0f);
+          for (int i = 0; i < 4; ++i)
+            if (live[i]) v |= (uint32_t)__ldg(cb + at + i) << (8 * i);
+          return v;
+        };
+        uint32_t lob[kChannels], hib[3];
+#pragma unroll
+        for (int k = 0; k < kChannels; ++k) {
+          const int c = c0 + k;
+          lob[k] = c < D ? four((c < 3 ? 2 * c + 1 : c + 3) * plane) : 0u;
+          if (k < 3) hib[k] = c < 3 && c < D ? four(2 * c * plane) : 0u;   // position: high bytes
+        }
+#pragma unroll
+        for (int k = 0; k < kChannels; ++k) {
+          const int c = c0 + k;
+          if (c >= D) break;
+          const float lo = s_lo[c], delta = s_delta[c];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint32_t q = (lob[k] >> (8 * i)) & 255u;
+            if (k < 3) q |= ((hib[k] >> (8 * i)) & 255u) << 8;
+            if (live[i]) dst[(int64_t)c * G + gidx[i]] = lpo_proxy(q, lo, delta);
           }
-          dst[gidx[i]] = lpo_proxy(q, lo, delta);
+        }
+      } else {
+#pragma unroll 4
+        for (int c = c0; c < min(c0 + kChannels, D); ++c) {
+          const float lo = s_lo[c], delta = s_delta[c];
+          const float *sc = reinterpret_cast<const float *>(src) + ((int64_t)f * D + c) * plane + pix;
+          float x[4] = {0.f, 0.f, 0.f, 0.f};
+          if (kVec) {
+            const float4 v = __ldg(reinterpret_cast<const float4 *>(sc));
+            x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (live[i]) x[i] = __ldg(sc + i);
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (live[i])
+              dst[(int64_t)c * G + gidx[i]] = lpo_proxy(lpo_code(x[i], lo, delta, c < 3 ? 65535.0f : 255.0f), lo, delta);
         }
       }
     }
   }
+}
+
+// One thread per group of four texels, one grid row per frame and channel group.
+dim3 gather_grid(int W, int H, int F, int D) {
+  const int64_t nq = (int64_t)((W + 3) / 4) * H;
+  const int64_t blocks = std::min<int64_t>(std::max<int64_t>(1, (nq + 255) / 256), 152 * 64);
+  return dim3((unsigned)blocks, (unsigned)std::min(std::max(F, 1) * ((D + kChannels - 1) / kChannels), 65535));
 }
 
 }  // namespace
@@ -280,17 +316,17 @@ extern "C" pk_status pk_atlas_gather_lpo(const pk_plan *p, const void *src, int3
   const int64_t nwords = (int64_t)((W + 31) / 32) * H;
   uint32_t *woff = at<uint32_t>(ws, p->ws.woff);
   pk_device_status *status = at<pk_device_status>(ws, p->ws.status);
-  k_word_scan<<<1, kScanThreads, 0, st>>>(occ, nwords, woff, status, p->N);
-  const int64_t nq = (int64_t)((W + 3) / 4) * H;
-  int blocks = (int)((nq + 255) / 256);
-  if (blocks > 152 * 64) blocks = 152 * 64;
-  if (blocks < 1) blocks = 1;
-  if (src_kind == PK_LPO_CODES)
-    k_gather_lpo<true><<<blocks, 256, 0, st>>>(src, lohi, occ, dyn, woff, W, H, p->F, p->D, p->N, soa, texel,
-                                               dynflag);
-  else
-    k_gather_lpo<false><<<blocks, 256, 0, st>>>(src, lohi, occ, dyn, woff, W, H, p->F, p->D, p->N, soa, texel,
-                                                dynflag);
+  launch_word_scan(occ, nwords, woff, status, p->N, st);
+  const dim3 blocks = gather_grid(W, H, p->F, p->D);
+  // four texels per load: whole groups per row, aligned planes (codes: any caller's pointer)
+  const bool vec = (W % 4) == 0 && (reinterpret_cast<uintptr_t>(src) & (src_kind == PK_LPO_CODES ? 3u : 15u)) == 0;
+#define PK_LPO(C, V) k_gather_lpo<C, V><<<blocks, 256, 0, st>>>(src, lohi, occ, dyn, woff, W, H, p->F, p->D, p->N, soa, texel, dynflag)
+  if (src_kind == PK_LPO_CODES) {
+    if (vec) PK_LPO(true, true); else PK_LPO(true, false);
+  } else {
+    if (vec) PK_LPO(false, true); else PK_LPO(false, false);
+  }
+#undef PK_LPO
   return check_launch();
 }
 
@@ -303,7 +339,7 @@ extern "C" pk_status pk_atlas_gather(const pk_plan *p, const void *atlas, const 
   const int64_t nwords = (int64_t)((W + 31) / 32) * H;
   uint32_t *woff = at<uint32_t>(ws, p->ws.woff);
   pk_device_status *status = at<pk_device_status>(ws, p->ws.status);
-  k_word_scan<<<1, kScanThreads, 0, st>>>(occ, nwords, woff, status, p->N);
+  launch_word_scan(occ, nwords, woff, status, p->N, st);
   const int64_t nq = (int64_t)((W + 3) / 4) * H;
   int blocks = (int)((nq + 255) / 256);
   if (blocks > 152 * 64) blocks = 152 * 64;
