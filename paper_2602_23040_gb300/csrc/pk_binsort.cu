@@ -235,12 +235,18 @@ __device__ __forceinline__ T block_excl_scan(T v, T &total, T *s) {
 __global__ __launch_bounds__(kThreads) void k_pair_count(const float *__restrict__ rec, int64_t pairs, int64_t N,
                                                          const DevView *__restrict__ views, int T, int mode,
                                                          uint32_t *__restrict__ cnt, uint4 *__restrict__ pinfo,
-                                                         uint32_t *__restrict__ zbits) {
+                                                         uint32_t *__restrict__ zbits,
+                                                         uint64_t *__restrict__ ranges, uint32_t n_ranges,
+                                                         uint32_t *abort_flag) {
   constexpr uint32_t kBalChunks = 64;   // a walk of up to 2,048 candidates keeps its ballots
   __shared__ WarpSplat s_ws[kWarps][32];
   __shared__ uint32_t s_bal[kWarps][kBalChunks];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t nwarps = (uint64_t)gridDim.x * kWarps;
+  // the call's first kernel also clears what the later ones add to
+  for (uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x; i < n_ranges; i += gridDim.x * (uint64_t)kThreads)
+    ranges[i] = 0ull;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *abort_flag = 0u;
   for (uint64_t w = blockIdx.x * (uint64_t)kWarps + warp; w * 32 < (uint64_t)pairs; w += nwarps) {
     const uint64_t p = w * 32 + lane;
     uint32_t ncand = 0;
@@ -360,58 +366,16 @@ __global__ __launch_bounds__(kThreads) void k_scan_reduce(Src src, const uint64_
   if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
-// Exclusive scan of the block sums (one block of 1024 threads, up to 4096
-// sums: kScanBlocks).  mode 0: compaction (total
-// = valid pairs); mode 1: emission offsets (total = entries, checked
-// against the capacity).
-__global__ __launch_bounds__(1024) void k_scan_top(uint64_t *__restrict__ bsum, int nb, int mode,
-                                                   uint64_t max_dups, DevCounters *ctr, pk_device_status *status) {
-  __shared__ uint64_t s[33];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // four consecutive block sums per thread (nb <= 4096)
-  uint64_t q[4], v = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    q[j] = 4 * tid + j < nb ? bsum[4 * tid + j] : 0;
-    v += q[j];
-  }
-  uint64_t incl = warp_incl_scan(v);
-  if (lane == 31) s[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    uint64_t w = s[lane];
-    uint64_t wi = warp_incl_scan(w);
-    s[lane] = wi - w;
-    if (lane == 31) s[32] = wi;
-  }
-  __syncthreads();
-  uint64_t run = s[warp] + incl - v;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (4 * tid + j < nb) bsum[4 * tid + j] = run;
-    run += q[j];
-  }
-  if (tid == 0) {
-    const uint64_t total = s[32];
-    ctr->scan_total = total;
-    if (mode == 0) {
-      ctr->n_valid = total;
-      status->valid_pairs = total;
-    } else {
-      status->dups_needed = total;
-      if (ctr->sort_abort) {   // a depth pass gave up: emit nothing
-        ctr->dups = 0;
-        status->dups = 0;
-      } else if (total > max_dups) {
-        ctr->dups = 0;
-        status->dups = 0;
-        atomicOr(&status->flags, PK_DEV_CAPACITY);
-      } else {
-        ctr->dups = total;
-        status->dups = total;
-      }
-    }
-  }
+// Items of the blocks before this one, from the block sums: every block of a
+// downsweep adds them up itself (at most 4096 sums, L2 hits), which takes
+// about a microsecond of each instead of a launch of one block between the
+// two sweeps (4.5 us).
+__device__ __forceinline__ uint64_t block_base(const uint64_t *__restrict__ bsum, uint64_t *s) {
+  uint64_t v = 0;
+  for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kThreads) v += __ldg(bsum + i);
+  uint64_t tot;
+  block_excl_scan<uint64_t>(v, tot, s);
+  return tot;
 }
 
 // Eight consecutive items of a u32 array from item i0 (a multiple of 8): two
@@ -435,12 +399,20 @@ static_assert(kScanItems == 8, "load8 takes a thread's scan items");
 __global__ __launch_bounds__(kThreads) void k_compact_down(const uint32_t *__restrict__ cnt,
                                                            const uint32_t *__restrict__ zbits, uint64_t n,
                                                            const uint64_t *__restrict__ bsum,
-                                                           uint32_t *__restrict__ zkey, uint32_t *__restrict__ pval) {
+                                                           uint32_t *__restrict__ zkey, uint32_t *__restrict__ pval,
+                                                           DevCounters *ctr, pk_device_status *status) {
   __shared__ uint32_t s[kWarps + 1];
+  __shared__ uint64_t s64[kWarps + 1];
   __shared__ uint32_t s_z[kScanTile], s_p[kScanTile];
   uint64_t b0, b1;
   chunk_of(n, gridDim.x, blockIdx.x, kScanTile, b0, b1);
-  uint32_t run = (uint32_t)bsum[blockIdx.x];   // valid pairs < 2^32
+  uint32_t run = (uint32_t)block_base(bsum, s64);   // valid pairs < 2^32
+  if (blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) {
+    const uint64_t total = run + bsum[blockIdx.x];
+    ctr->scan_total = total;
+    ctr->n_valid = total;
+    status->valid_pairs = total;
+  }
   for (uint64_t base = b0; base < b1; base += kScanTile) {
     const uint64_t i0 = base + (uint64_t)threadIdx.x * kScanItems;
     uint32_t cv[8], zv[8], c = 0;
@@ -504,15 +476,30 @@ __global__ __launch_bounds__(kThreads) void k_reduce_sorted(const uint32_t *__re
 
 // Down-sweep of the emission-offset scan: offs[i] = entries before pair i
 // (64-bit: the entries of a launch may pass 2^32), from the gathered counts.
+// The last block checks the total against the capacity.
 __global__ __launch_bounds__(kThreads) void k_offsets_down(const uint32_t *__restrict__ csorted,
                                                            const uint64_t *n_dev, const uint64_t *__restrict__ bsum,
-                                                           const DevCounters *ctr, uint64_t *__restrict__ offs) {
+                                                           uint64_t max_dups, DevCounters *ctr,
+                                                           pk_device_status *status, uint64_t *__restrict__ offs) {
   __shared__ uint64_t s[kWarps + 1];
-  if (ctr->dups == 0) return;   // overflow (or nothing): nothing will be emitted
   const uint64_t n = *n_dev;
   uint64_t b0, b1;
   chunk_of(n, gridDim.x, blockIdx.x, kScanTile, b0, b1);
-  uint64_t run = bsum[blockIdx.x];
+  uint64_t run = block_base(bsum, s);
+  if (blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) {
+    const uint64_t total = run + bsum[blockIdx.x];
+    ctr->scan_total = total;
+    status->dups_needed = total;
+    uint64_t dups = total;
+    if (ctr->sort_abort) {   // a depth pass gave up: emit nothing
+      dups = 0;
+    } else if (total > max_dups) {
+      dups = 0;
+      atomicOr(&status->flags, PK_DEV_CAPACITY);
+    }
+    ctr->dups = dups;
+    status->dups = dups;
+  }
   for (uint64_t base = b0; base < b1; base += kScanTile) {
     const uint64_t i0 = base + (uint64_t)threadIdx.x * kScanItems;
     uint32_t v[8];
@@ -557,16 +544,22 @@ struct SegSpec {
   const uint64_t *seg;
 };
 
+// part: the block's part of its segment (or of the array); sbase: the
+// segment's first item.
 __device__ __forceinline__ void radix_chunk(const SegSpec &sp, uint64_t n, int tile, uint64_t &b0, uint64_t &b1,
-                                            uint32_t &hbase, uint32_t &hstride) {
+                                            uint32_t &hbase, uint32_t &hstride, uint32_t &part, uint64_t &sbase) {
   if (!sp.tab) {
     chunk_of(n, gridDim.x, blockIdx.x, tile, b0, b1);
     hbase = blockIdx.x;
     hstride = gridDim.x;
+    part = blockIdx.x;
+    sbase = 0;
     return;
   }
   const int4 t = sp.tab[blockIdx.x];
   const uint64_t s0 = sp.seg[t.x], s1 = sp.seg[t.x + 1];
+  part = (uint32_t)t.y;
+  sbase = s0;
   chunk_of(s1 - s0, t.z, t.y, tile, b0, b1);
   b0 += s0;
   b1 += s0;
@@ -591,18 +584,38 @@ struct Radix {
 };
 constexpr int kPairItems = 12, kEntryItems = 8;
 
+// Blocks of a pass: at most one per tile of keys.  An unsegmented pass takes
+// one resident wave at most, whose parts are equal; a segmented one up to
+// kSegWaves waves, since its parts are whole numbers per view and one wave
+// shared among 208 views left the small views' single blocks with twice the
+// keys of the large views' (the tile passes of the 4 x 52-view sequence, of
+// 71 ms in all: 6.8 + 5.1 ms and 1.7 of upsweeps, now 3.6 + 2.9 and 0.9).
+constexpr int kSegWaves = 4;
+// Where a downsweep block takes the positions of its digits from: kScan, the
+// counters scanned by two launches; kDirect, with few parts per segment, the
+// segment's counts added up by every block itself (coalesced: the counters
+// lie [part][digit] then), which saves those launches at up to kDirectLoads
+// parts x blocks (2 KB each, L2 hits); kSolo, where every segment is one
+// block of at most kSoloTiles tiles, its own count of its keys, with no
+// upsweep either (the small sorts are bound by launches, 7 to 10 us of host
+// time each in an eager step).
+enum DigitBase { kScan, kDirect, kSolo };
+constexpr int kDirectParts = 64, kDirectLoads = 65536, kSoloTiles = 2;
+
 template <int RB, int IT>
 __global__ __launch_bounds__(kThreads) void k_radix_upsweep(const uint32_t *__restrict__ keys,
                                                             const uint64_t *n_dev, uint64_t n_host, int shift,
-                                                            uint32_t mask, uint64_t *__restrict__ hist, SegSpec sp) {
+                                                            uint32_t mask, uint64_t *__restrict__ hist,
+                                                            DigitBase base, SegSpec sp) {
   using C = Radix<RB, IT>;
   __shared__ uint32_t s_cnt[C::kCopies][C::kR];   // private digit counts
   for (int i = threadIdx.x; i < C::kCopies * C::kR; i += kThreads) (&s_cnt[0][0])[i] = 0;
   __syncthreads();
   const uint64_t n = load_n(n_dev, n_host);
   uint64_t b0, b1;
-  uint32_t hbase, hstride;
-  radix_chunk(sp, n, C::kTile, b0, b1, hbase, hstride);
+  uint32_t hbase, hstride, part;
+  uint64_t sbase;
+  radix_chunk(sp, n, C::kTile, b0, b1, hbase, hstride, part, sbase);
   uint32_t *cw = s_cnt[(threadIdx.x >> 5) % C::kCopies];
   // up to 3 keys before the first 16-byte boundary (segments start anywhere)
   const uint64_t a0 = min(b1, (b0 + 3) & ~uint64_t(3));
@@ -633,7 +646,7 @@ __global__ __launch_bounds__(kThreads) void k_radix_upsweep(const uint32_t *__re
     uint32_t t = 0;
 #pragma unroll
     for (int w = 0; w < C::kCopies; ++w) t += s_cnt[w][d];
-    hist[hbase + (size_t)d * hstride] = t;
+    hist[base == kDirect ? hbase - part + (size_t)part * C::kR + d : hbase + (size_t)d * hstride] = t;
   }
 }
 
@@ -765,7 +778,7 @@ __global__ __launch_bounds__(kThreads, (Radix<RB, IT>::kMinBlocks)) void k_radix
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const uint64_t *n_dev, uint64_t n_host, int shift, uint32_t mask,
     const uint64_t *__restrict__ hist, pk_device_status *status, SegSpec sp, uint32_t *abort_flag,
-    uint32_t first_polls, bool try_single, Unpack up) {
+    uint32_t first_polls, bool try_single, DigitBase dbase, Unpack up) {
   using C = Radix<RB, IT>;
   constexpr bool kV = kMode == 0, kLast = kMode == 2;
   constexpr int kTile = C::kTile;
@@ -779,11 +792,13 @@ __global__ __launch_bounds__(kThreads, (Radix<RB, IT>::kMinBlocks)) void k_radix
   uint64_t *s_bar = reinterpret_cast<uint64_t *>(
       (reinterpret_cast<uintptr_t>(s_scan + kWarps + 1) + 7) & ~uintptr_t(7));      // [2]
   __shared__ int s_abort;
+  __shared__ uint64_t s_dir[kWarps + 1];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint64_t n = load_n(n_dev, n_host);
   uint64_t b0, b1;
-  uint32_t hbase, hstride;
-  radix_chunk(sp, n, kTile, b0, b1, hbase, hstride);
+  uint32_t hbase, hstride, part;
+  uint64_t sbase;
+  radix_chunk(sp, n, kTile, b0, b1, hbase, hstride, part, sbase);
   if (b1 - b0 > 0xffffffffull) {   // a block's digit counts are 32-bit: give the call up
     if (tid == 0) {
       atomicOr(&status->flags, PK_DEV_BOUNDS);
@@ -791,7 +806,38 @@ __global__ __launch_bounds__(kThreads, (Radix<RB, IT>::kMinBlocks)) void k_radix
     }
     return;
   }
-  for (int d = tid; d < C::kR; d += kThreads) s_gbase[d] = hist[hbase + (size_t)d * hstride];
+  if (dbase == kScan) {
+    for (int d = tid; d < C::kR; d += kThreads) s_gbase[d] = hist[hbase + (size_t)d * hstride];
+  } else {
+    if (dbase == kSolo) {   // this block's keys are its segment's: count them here
+      for (int d = tid; d < C::kR; d += kThreads) s_start[d] = 0u;
+      __syncthreads();
+      for (uint64_t i = b0 + tid; i < b1; i += kThreads) atomicAdd(&s_start[(__ldg(kin + i) >> shift) & mask], 1u);
+      __syncthreads();
+    }
+    const uint64_t *h = hist + (hbase - part);
+    uint64_t before[C::kPerThread], sum = 0;
+#pragma unroll
+    for (int u = 0; u < C::kPerThread; ++u) {
+      const int d = tid * C::kPerThread + u;
+      uint64_t pre = sum;
+      if (dbase == kSolo) {
+        sum += s_start[d];
+      } else {
+#pragma unroll 8
+        for (uint32_t j = 0; j < hstride; ++j) {
+          const uint64_t c = h[(size_t)j * C::kR + d];
+          sum += c;
+          if (j < part) pre += c;
+        }
+      }
+      before[u] = pre;
+    }
+    uint64_t tot;
+    const uint64_t ex = sbase + block_excl_scan<uint64_t>(sum, tot, s_dir);
+#pragma unroll
+    for (int u = 0; u < C::kPerThread; ++u) s_gbase[tid * C::kPerThread + u] = ex + before[u];
+  }
   const int ntile = (int)((b1 - b0 + kTile - 1) / kTile);
   // last packed pass: the block's view (segmented) turns local ids global
   uint32_t tile0 = 0, tile1 = up.n_tiles;
@@ -1220,35 +1266,40 @@ __global__ __launch_bounds__(kThreads) void k_view_segments(const uint32_t *__re
 template <int RB, int IT, int kMode>
 pk_status radix_pass_rb(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
                         const uint64_t *n_dev, uint64_t n_host, int shift, int bits, uint64_t *hist, int nblocks,
-                        uint64_t *csum, pk_device_status *status, SegSpec sp, uint32_t *abort_flag,
+                        DigitBase dbase, uint64_t *csum, pk_device_status *status, SegSpec sp, uint32_t *abort_flag,
                         uint32_t first_polls, bool try_single, const Unpack &up, cudaStream_t st) {
   using C = Radix<RB, IT>;
   if (cudaFuncSetAttribute(k_radix_downsweep<RB, IT, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)Down<RB, IT>::kSmem) != cudaSuccess)
     return PK_ERR_CUDA;
   const uint32_t mask = (1u << bits) - 1u;
-  k_radix_upsweep<RB, IT><<<nblocks, kThreads, 0, st>>>(kin, n_dev, n_host, shift, mask, hist, sp);
-  const int count = C::kR * nblocks, nchunks = (count + kHistChunk - 1) / kHistChunk;
-  k_radix_chunk_sums<<<nchunks, 1024, 0, st>>>(hist, count, csum);
-  k_radix_scan_chunks<<<nchunks, 1024, 0, st>>>(hist, count, csum);
+  if (dbase != kSolo)
+    k_radix_upsweep<RB, IT><<<nblocks, kThreads, 0, st>>>(kin, n_dev, n_host, shift, mask, hist, dbase, sp);
+  if (dbase == kScan) {
+    const int count = C::kR * nblocks, nchunks = (count + kHistChunk - 1) / kHistChunk;
+    k_radix_chunk_sums<<<nchunks, 1024, 0, st>>>(hist, count, csum);
+    k_radix_scan_chunks<<<nchunks, 1024, 0, st>>>(hist, count, csum);
+  }
   k_radix_downsweep<RB, IT, kMode><<<nblocks, kThreads, Down<RB, IT>::kSmem, st>>>(
-      kin, vin, kout, vout, n_dev, n_host, shift, mask, hist, status, sp, abort_flag, first_polls, try_single, up);
+      kin, vin, kout, vout, n_dev, n_host, shift, mask, hist, status, sp, abort_flag, first_polls, try_single, dbase,
+      up);
   return check_launch();
 }
 
 // One stable pass over key bits [shift, shift + bits), bits <= 8, over the
-// depth-sorted pairs (pair_blocks() blocks) or over the entries
-// (sort_blocks() blocks, or the segmented table's), with digits of up to
+// depth-sorted pairs or over the entries (nblocks blocks: part_count() of
+// the array, or the segmented table's), with digits of up to
 // rb = 8 or 11 bits (pk_options.sort_bits_*: wider digits take fewer passes
 // but run fewer blocks per SM and scatter into more runs).  vin == nullptr:
 // packed entries, keys only; then up.ranges != nullptr marks the last pass.
 pk_status radix_pass(bool entries, int rb, const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
                      const uint64_t *n_dev, uint64_t n_host, int shift, int bits, uint64_t *hist, int nblocks,
-                     uint64_t *csum, pk_device_status *status, uint32_t *abort_flag, uint32_t first_polls,
+                     DigitBase dbase, uint64_t *csum, pk_device_status *status, uint32_t *abort_flag, uint32_t first_polls,
                      bool try_single, cudaStream_t st, SegSpec sp = SegSpec{nullptr, nullptr},
                      Unpack up = Unpack{}) {
 #define PK_PASS(RB, IT, M)                                                                                        \
-  return radix_pass_rb<RB, IT, M>(kin, vin, kout, vout, n_dev, n_host, shift, bits, hist, nblocks, csum, status, \
+  return radix_pass_rb<RB, IT, M>(kin, vin, kout, vout, n_dev, n_host, shift, bits, hist, nblocks, dbase, csum,   \
+                                  status,                                                                   \
                                   sp, abort_flag, first_polls, try_single, up, st)
   if (entries) {
     if (!vin && up.ranges) {
@@ -1274,59 +1325,78 @@ int sm_count() {
   return std::max(1, sms);
 }
 
-// Blocks of the pair passes: resident ones, within the histogram.
-int pair_blocks(int rb) {
-  const int per_sm = rb > 8 ? Radix<11, kPairItems>::kMinBlocks : Radix<8, kPairItems>::kMinBlocks;
-  return std::max(1, std::min(kSortBlocks, per_sm * sm_count()));
+// Blocks of an unsegmented pass over at most `items` pairs or entries, or
+// (waves > 1) the blocks that a segmented one shares out.
+int part_count(bool entries, int rb, uint64_t items, int waves, int cap) {
+  const int tile = kThreads * (entries ? kEntryItems : kPairItems);
+  const int per_sm = entries ? (rb > 8 ? Radix<11, kEntryItems>::kMinBlocks : Radix<8, kEntryItems>::kMinBlocks)
+                             : (rb > 8 ? Radix<11, kPairItems>::kMinBlocks : Radix<8, kPairItems>::kMinBlocks);
+  if (waves == 1 && items <= (uint64_t)tile * kSoloTiles) return 1;
+  const uint64_t useful = (items + (uint64_t)tile - 1) / (uint64_t)tile;
+  const uint64_t most = (uint64_t)std::min(cap, waves * per_sm * sm_count());
+  return (int)std::max<uint64_t>(1, std::min(useful, most));
 }
 
-}  // namespace
-
-// Blocks of the entry passes on this device.
-int pk::sort_blocks(int rb) {
-  // the entry passes' resident blocks, leaving the histogram room for the
-  // segmented table's one extra block per view
-  const int per_sm = rb > 8 ? Radix<11, kEntryItems>::kMinBlocks : Radix<8, kEntryItems>::kMinBlocks;
-  return std::max(1, std::min(kSortBlocks - 128, per_sm * sm_count()));
+// How a pass of `blocks` blocks, at most `parts` per segment of at most
+// `items` keys, finds its digits' positions.
+int digit_base(bool entries, int blocks, int parts, uint64_t items) {
+  const uint64_t tile = (uint64_t)kThreads * (entries ? kEntryItems : kPairItems);
+  if (parts == 1 && items <= tile * kSoloTiles) return kSolo;
+  return parts <= kDirectParts && (int64_t)blocks * parts <= kDirectLoads ? kDirect : kScan;
 }
-
-namespace {
 
 // Block table of a segmented sort: per view a share of `nblocks`
 // proportional to weight(v) (at least one), each {view, part, parts, first
 // histogram counter}.  Returns the number of blocks, or 0 when the views do
-// not fit the histogram.
+// not fit the histogram; *most = the largest number of parts.
 template <typename Weight>
-int share_blocks(int V, int nblocks, int rb, const Weight &weight, int4 *tab) {
+int share_blocks(int V, int nblocks, int cap, int rb, const Weight &weight, int4 *tab, int *most) {
   int64_t total = 0;
   for (int v = 0; v < V; ++v) total += weight(v);
   int nb = 0;
+  *most = 0;
   for (int v = 0; v < V; ++v) {
     const int parts = std::max<int>(1, (int)((int64_t)nblocks * weight(v) / std::max<int64_t>(1, total)));
-    if (nb + parts > kSortBlocks) return 0;
+    if (nb + parts > cap) return 0;
     for (int j = 0; j < parts; ++j) tab[nb + j] = make_int4(v, j, parts, (1 << rb) * nb);
     nb += parts;
+    *most = std::max(*most, parts);
   }
   return nb;
 }
 
 }  // namespace
 
-// The tile passes' table (shares by tiles) and the depth passes' (equal
-// shares: every view has N pairs at most); false when the plan sorts
-// unsegmented (one view, or too many views for the histogram).
-bool pk::seg_tables(const pk_plan *p, int4 *tab, int *ntile, int *npair) {
-  *ntile = *npair = 0;
-  if (p->V < 2) return false;
+// The tile passes' table (shares by tiles; tab[0, cap)) and the depth
+// passes' (equal shares: every view has N pairs at most; tab[cap, 2 cap));
+// `false` in the result's ntile: the plan sorts unsegmented (one view, or too
+// many views for the histogram).
+pk::SortBlocks pk::sort_layout(const pk_plan *p, int cap, int4 *tab) {
   const int rt = p->opts.sort_bits_tile, rd = p->opts.sort_bits_depth;
-  const int nt = share_blocks(p->V, sort_blocks(rt), rt,
-                              [&](int v) { return (int64_t)p->h_views[v].tiles_x * p->h_views[v].tiles_y; },
-                              tab);
-  const int np = share_blocks(p->V, pair_blocks(rd), rd, [](int) { return int64_t(1); }, tab + kSortBlocks);
-  if (nt == 0 || np == 0) return false;
-  *ntile = nt;
-  *npair = np;
-  return true;
+  const uint64_t pairs = (uint64_t)p->pairs, maxd = p->max_dups;
+  SortBlocks b{};
+  if (p->V >= 2) {
+    // room for the one block a view takes at least
+    const int room = std::max(1, cap - std::min(p->V, cap / 2));
+    int mt = 0, mp = 0;
+    const int nt = share_blocks(p->V, part_count(true, rt, maxd, kSegWaves, room), cap, rt,
+                                [&](int v) { return (int64_t)p->h_views[v].tiles_x * p->h_views[v].tiles_y; }, tab, &mt);
+    const int np = share_blocks(p->V, part_count(false, rd, pairs, kSegWaves, room), cap, rd,
+                                [](int) { return int64_t(1); }, tab + cap, &mp);
+    if (nt != 0 && np != 0) {
+      b.seg = true;
+      b.ntile = nt;
+      b.npair = np;
+      b.tile_base = digit_base(true, nt, mt, maxd);
+      b.pair_base = digit_base(false, np, mp, (uint64_t)p->N);
+      return b;
+    }
+  }
+  b.ntile = part_count(true, rt, maxd, 1, cap);
+  b.npair = part_count(false, rd, pairs, 1, cap);
+  b.tile_base = digit_base(true, b.ntile, b.ntile, maxd);
+  b.pair_base = digit_base(false, b.npair, b.npair, pairs);
+  return b;
 }
 
 namespace {
@@ -1376,23 +1446,20 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   // segmented sorts (V >= 2): the depth passes sort each view's pairs in
   // place, the tile passes each view's entries on per-view local tile ids
   int4 tab_host[2 * kSortBlocks];
-  int nseg = 0, npseg = 0;
-  const bool seg = seg_tables(p, tab_host, &nseg, &npseg);
+  const SortBlocks blk = sort_layout(p, L.sort_cap, tab_host);
+  const bool seg = blk.seg;
   const int4 *tab = at<int4>(ws, L.sblk);
   uint64_t *vseg = at<uint64_t>(ws, L.vseg), *pseg = vseg + (p->V + 1);
 
-  pk_status ze = zero_async({{tile_ranges, sizeof(uint64_t) * 2 * (size_t)p->n_tiles},
-                             {ctr, pairs == 0 ? sizeof(DevCounters) : 0},
-                             {&ctr->sort_abort, pairs == 0 ? 0 : sizeof(uint32_t)}},
-                            st);
-  if (ze != PK_OK || pairs == 0) return ze;
+  if (pairs == 0)
+    return zero_async({{tile_ranges, sizeof(uint64_t) * 2 * (size_t)p->n_tiles}, {ctr, sizeof(DevCounters)}}, st);
   const int cblocks = (int)std::min<uint64_t>((pairs + kThreads - 1) / kThreads, 152 * 16);
   k_pair_count<<<cblocks, kThreads, 0, st>>>(records, p->pairs, p->N, views, p->T, p->opts.bin_mode, cnt, pinfo,
-                                              zk[1]);
+                                              zk[1], tile_ranges, 2u * (uint32_t)p->n_tiles, &ctr->sort_abort);
   // compaction of the pairs that touch a tile, keyed by depth bits
-  k_scan_reduce<SrcValid><<<kScanBlocks, kThreads, 0, st>>>(SrcValid{cnt}, nullptr, pairs, bsum);
-  k_scan_top<<<1, 1024, 0, st>>>(bsum, kScanBlocks, 0, maxd, ctr, status);
-  k_compact_down<<<kScanBlocks, kThreads, 0, st>>>(cnt, zk[1], pairs, bsum, zk[0], pv[0]);
+  const int sblocks = (int)std::min<uint64_t>((pairs + kScanTile - 1) / kScanTile, kScanBlocks);
+  k_scan_reduce<SrcValid><<<sblocks, kThreads, 0, st>>>(SrcValid{cnt}, nullptr, pairs, bsum);
+  k_compact_down<<<sblocks, kThreads, 0, st>>>(cnt, zk[1], pairs, bsum, zk[0], pv[0], ctr, status);
   // depth sort of the pairs: stable passes over the 32 bits of z; the
   // compaction kept the (view, Gaussian) order, so sorting inside each
   // view's segment leaves the pairs in (view, depth) order
@@ -1400,7 +1467,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   if (seg) {
     k_view_segments<false><<<(p->V + kThreads) / kThreads, kThreads, 0, st>>>(pv[0], nullptr, ctr, (uint32_t)p->N,
                                                                             p->V, pseg);
-    psp = SegSpec{tab + kSortBlocks, pseg};
+    psp = SegSpec{tab + L.sort_cap, pseg};
   }
   pk_status e;
   int widths[8];
@@ -1409,7 +1476,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   for (int pass = 0; pass < np; ++pass) {
     const int a = pass & 1, b = a ^ 1;
     if ((e = radix_pass(false, rd, zk[a], pv[a], zk[b], pv[b], n_valid, 0, shift, widths[pass], hist,
-                        seg ? npseg : pair_blocks(rd), bsum, status, &ctr->sort_abort, p->first_polls,
+                        blk.npair, (DigitBase)blk.pair_base, bsum, status, &ctr->sort_abort, p->first_polls,
                         pass == np - 1, st, psp)) != PK_OK)
       return e;
     shift += widths[pass];
@@ -1417,19 +1484,16 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   const uint32_t *pval = pv[np & 1];
   // emission offsets in (view,) depth order, capacity check
   uint32_t *csorted = zk[1];   // the depth keys are spent: their buffer takes the gathered counts
-  k_reduce_sorted<<<kScanBlocks, kThreads, 0, st>>>(cnt, pval, pairs, n_valid, csorted, bsum);
-  k_scan_top<<<1, 1024, 0, st>>>(bsum, kScanBlocks, 1, maxd, ctr, status);
-  k_offsets_down<<<kScanBlocks, kThreads, 0, st>>>(csorted, n_valid, bsum, ctr, offs);
+  k_reduce_sorted<<<sblocks, kThreads, 0, st>>>(cnt, pval, pairs, n_valid, csorted, bsum);
+  k_offsets_down<<<sblocks, kThreads, 0, st>>>(csorted, n_valid, bsum, maxd, ctr, status, offs);
   // emission and the stable tile sort; the last pass lands in sorted_vals
   int key_bits = p->tile_bits;
   SegSpec sp{nullptr, nullptr};
-  int nblocks = sort_blocks(rt);
   if (seg) {
     key_bits = local_tile_bits(p);
     k_view_segments<true><<<(p->V + kThreads) / kThreads, kThreads, 0, st>>>(pval, offs, ctr, (uint32_t)p->N, p->V,
                                                                           vseg);
     sp = SegSpec{tab, vseg};
-    nblocks = nseg;
   }
   // Packed entries when the tile id and the pair index fit one word
   // together (both local to the view in a segmented sort; at the 52-view
@@ -1460,11 +1524,12 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
     shift -= widths[pass];
     if (packed)
       e = radix_pass(true, rt, kbuf[a], nullptr, last ? nullptr : kbuf[b], last ? sorted_vals : nullptr, &ctr->dups,
-                     0, shift, widths[pass], hist, nblocks, bsum, status, &ctr->sort_abort, p->first_polls, false,
+                     0, shift, widths[pass], hist, blk.ntile, (DigitBase)blk.tile_base, bsum, status, &ctr->sort_abort,
+                     p->first_polls, false,
                      st, sp, last ? up : Unpack{});
     else
-      e = radix_pass(true, rt, kbuf[a], vbuf[a], kbuf[b], vbuf[b], &ctr->dups, 0, shift, widths[pass], hist, nblocks,
-                     bsum, status, &ctr->sort_abort, p->first_polls, false, st, sp);
+      e = radix_pass(true, rt, kbuf[a], vbuf[a], kbuf[b], vbuf[b], &ctr->dups, 0, shift, widths[pass], hist, blk.ntile,
+                     (DigitBase)blk.tile_base, bsum, status, &ctr->sort_abort, p->first_polls, false, st, sp);
     if (e != PK_OK) return e;
   }
   if (packed)
@@ -1478,21 +1543,22 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
 
 }  // namespace
 
-// Mirrors the launches of bin_and_sort_impl: zeroing, count, scan (2),
-// compaction, [pair segments], the depth passes, offsets (3), [entry
-// segments], emission, the tile passes, ranges; 4 kernels per radix pass.
+// Mirrors the launches of bin_and_sort_impl: count, scan, compaction, [pair
+// segments], the depth passes, offsets (2), [entry segments], emission, the
+// tile passes, ranges; 1, 2 or 4 kernels per radix pass (DigitBase).
 int pk::bin_kernel_count(const pk_plan *p) {
   if (!p) return 0;
   if (p->pairs == 0) return 1;
   int4 tab[2 * kSortBlocks];
-  int nt = 0, np = 0;
-  const bool seg = seg_tables(p, tab, &nt, &np);
+  const SortBlocks blk = sort_layout(p, p->ws.sort_cap, tab);
   int widths[8];
-  int passes = radix_plan(32, p->opts.sort_bits_depth, widths);
-  int kernels = 1 + 4 + 3 + 1 + 1;
-  if (seg) kernels += 2;   // the pairs' and the entries' view segments
-  passes += radix_plan(seg ? local_tile_bits(p) : p->tile_bits, p->opts.sort_bits_tile, widths);
-  return kernels + 4 * passes;
+  auto launches = [](int base) { return base == kScan ? 4 : base == kDirect ? 2 : 1; };
+  int kernels = 3 + 2 + 1 + 1;
+  if (blk.seg) kernels += 2;   // the pairs' and the entries' view segments
+  kernels += radix_plan(32, p->opts.sort_bits_depth, widths) * launches(blk.pair_base);
+  kernels += radix_plan(blk.seg ? local_tile_bits(p) : p->tile_bits, p->opts.sort_bits_tile, widths) *
+             launches(blk.tile_base);
+  return kernels;
 }
 
 extern "C" pk_status pk_bin_and_sort(const pk_plan *p, const float *records, uint32_t *sorted_vals,
@@ -1521,6 +1587,7 @@ extern "C" pk_status pk_bin_and_sort(const pk_plan *p, const float *records, uin
 
 namespace {
 
+constexpr int kStaticSortBlocks = 768;   // radix blocks that the static array holds counters for
 constexpr size_t kStaticScratchBytes = size_t(64) << 20;   // 64 MiB, held by every GPU that loads the library
 constexpr int kMaxDevices = 64;
 __device__ __align__(256) unsigned char g_bin_scratch[kStaticScratchBytes];
@@ -1601,7 +1668,8 @@ extern "C" pk_status pk_bin_and_sort_noalloc(const pk_plan *p, const float *reco
   L.counters = take(sizeof(DevCounters));
   L.views = take(sizeof(DevView) * p->V);
   L.toff = take(sizeof(uint32_t) * (p->V + 1));
-  L.sblk = take(sizeof(int4) * 2 * kSortBlocks);
+  L.sort_cap = kStaticSortBlocks;
+  L.sblk = take(sizeof(int4) * 2 * kStaticSortBlocks);
   L.vseg = take(sizeof(uint64_t) * 2 * (p->V + 1));
   L.pair_cnt = take(sizeof(uint32_t) * pairs);
   L.zkey0 = take(sizeof(uint32_t) * pairs);
@@ -1613,7 +1681,7 @@ extern "C" pk_status pk_bin_and_sort_noalloc(const pk_plan *p, const float *reco
   L.blocksums = take(sizeof(uint64_t) * (kScanBlocks + 1));
   // digit counters of the widest radix pass of the plan's two sorts
   L.hist = take(sizeof(uint64_t) * (size_t(1) << std::max(p->opts.sort_bits_tile, p->opts.sort_bits_depth)) *
-                kSortBlocks);
+                kStaticSortBlocks);
   L.dkey0 = take(sizeof(uint32_t) * maxd);
   L.dkey1 = take(sizeof(uint32_t) * maxd);
   L.dval = take(sizeof(uint32_t) * maxd);
@@ -1628,9 +1696,8 @@ extern "C" pk_status pk_bin_and_sort_noalloc(const pk_plan *p, const float *reco
   if ((e = zero_async({{at<char>(ws, L.status), L.views - L.status}}, st)) != PK_OK) return e;
   if ((e = put_words(at<char>(ws, L.views), p->h_views, sizeof(DevView) * p->V, st)) != PK_OK) return e;
   if ((e = put_words(at<char>(ws, L.toff), p->h_toff, sizeof(uint32_t) * (p->V + 1), st)) != PK_OK) return e;
-  int4 tab[2 * kSortBlocks] = {};
-  int nt = 0, np = 0;
-  if (seg_tables(p, tab, &nt, &np) && (e = put_words(at<char>(ws, L.sblk), tab, sizeof(tab), st)) != PK_OK)
+  int4 tab[2 * kStaticSortBlocks] = {};
+  if (sort_layout(p, L.sort_cap, tab).seg && (e = put_words(at<char>(ws, L.sblk), tab, sizeof(tab), st)) != PK_OK)
     return e;
   if ((e = bin_and_sort_impl(p, L, ws, records, sorted_vals, tile_ranges, maxd, st)) != PK_OK) return e;
   const DevCounters *ctr = at<DevCounters>(ws, L.counters);

@@ -30,7 +30,7 @@ constexpr float kInvExpScale = -1.38629436111989061f;   // 1 / kExpScale = -2 ln
 
 // Fixed grid sizes of the device-count-driven kernels (scan, radix sort).
 constexpr int kScanBlocks = 4096;
-constexpr int kSortBlocks = 768;      // most radix blocks of one pass (histogram capacity)
+constexpr int kSortBlocks = 2560;     // most radix blocks of one pass (histogram capacity)
 constexpr int kMaxRadixBits = 11;     // widest radix digit (pk_options.sort_bits_*: 8 or 11)
 constexpr uint64_t kMaxEntries = uint64_t(1) << 35;   // most (pair, tile) entries of a plan
 
@@ -69,8 +69,9 @@ struct WsLayout {
   size_t pair_cnt, zkey0, zkey1, pval0, pval1, offs, rmask;   // rmask: per pair {mask (2 words), rectangle (2)}
   size_t blocksums, hist;
   size_t dkey0, dkey1, dval;
-  size_t sblk, vseg;       // segmented sorts: block tables [2][kSortBlocks] int4 (tile passes, depth
+  size_t sblk, vseg;       // segmented sorts: block tables [2][sort_cap] int4 (tile passes, depth
                            // passes), view starts [2][V + 1] (entries, pairs)
+  int sort_cap;            // most radix blocks of one pass (counters in hist)
   size_t mask_tmp;         // one motion mask's worth of words (dilation scratch)
   size_t mask_coarse;      // per view, one bit per 32 x 32-pixel block: any moving pixel
   size_t total;
@@ -110,12 +111,15 @@ bool aligned16(const void *p);
 // Zero up to four (pointer, bytes) ranges with one kernel (4-byte aligned
 // pointers, sizes multiples of 4 bytes).
 pk_status zero_async(std::initializer_list<std::pair<void *, size_t>> spans, cudaStream_t st);
-// Radix blocks of the entry passes on the current device, and the block
-// tables of the segmented (per-view) sorts: tab[0, kSortBlocks) for the
-// tile passes, tab[kSortBlocks, 2 kSortBlocks) for the depth passes
-// (pk_binsort.cu); false = the plan sorts unsegmented.
-int sort_blocks(int rb);
-bool seg_tables(const pk_plan *p, int4 *tab, int *ntile, int *npair);
+// Radix blocks of the tile and depth passes on the current device, whether
+// they sort view by view (seg; then tab[0, cap) is the tile passes' block
+// table and tab[cap, 2 cap) the depth passes') and where their downsweeps take
+// the digit positions from (DigitBase, pk_binsort.cu).
+struct SortBlocks {
+  bool seg;
+  int ntile, npair, tile_base, pair_base;
+};
+SortBlocks sort_layout(const pk_plan *p, int cap, int4 *tab);
 // Kernels one pk_bin_and_sort call launches for this plan on this device.
 int bin_kernel_count(const pk_plan *p);
 

@@ -326,6 +326,7 @@ extern "C" pk_status pk_plan_create(const pk_atlas_desc *desc, const pk_view *vi
   L.dkey0 = take(sizeof(uint32_t) * maxd);
   L.dkey1 = take(sizeof(uint32_t) * maxd);
   L.dval = take(sizeof(uint32_t) * maxd);
+  L.sort_cap = kSortBlocks;
   L.sblk = take(sizeof(int4) * 2 * kSortBlocks);
   L.vseg = take(sizeof(uint64_t) * 2 * (V + 1));
   L.mask_tmp = take(sizeof(uint32_t) * (size_t)p->mask_words);
@@ -386,8 +387,7 @@ extern "C" pk_status pk_workspace_init(const pk_plan *p, void *ws, pk_stream_t s
     return PK_ERR_CUDA;
   // block tables of the segmented sorts (for this device's SM count)
   int4 *tab = const_cast<pk_plan *>(p)->h_segtab;
-  int nt = 0, np = 0;
-  if (seg_tables(p, tab, &nt, &np) &&
+  if (sort_layout(p, kSortBlocks, tab).seg &&
       cudaMemcpyAsync(at<char>(ws, L.sblk), tab, sizeof(p->h_segtab), cudaMemcpyHostToDevice, st) != cudaSuccess)
     return PK_ERR_CUDA;
   // pageable sources: make sure the copies are done before the plan may go away
@@ -508,8 +508,7 @@ extern "C" pk_status pk_autotune(pk_plan *p, const float *records, uint32_t *sor
   // whole call; the lists do not depend on them.  The segmented sorts'
   // block tables depend on the widths and are uploaded again.
   auto upload_tables = [&]() -> pk_status {
-    int nt = 0, np = 0;
-    if (seg_tables(p, p->h_segtab, &nt, &np) &&
+    if (sort_layout(p, kSortBlocks, p->h_segtab).seg &&
         cudaMemcpyAsync(at<char>(ws, p->ws.sblk), p->h_segtab, sizeof(p->h_segtab), cudaMemcpyHostToDevice, st) !=
             cudaSuccess)
       return PK_ERR_CUDA;
