@@ -63,7 +63,7 @@ __device__ __forceinline__ int view_of_tile(const uint32_t *__restrict__ toff, i
 struct Staged {
   float4 *a;     // m_x, m_y, A = k conic_a, B = 2 k conic_b      (k = -log2(e) / 2)
   float4 *b;     // C = k conic_c, -opacity, red, green
-  float4 *c;     // blue, pair index (bits), pcut, 0
+  float4 *c;     // blue, pair index (bits), pcut, -1 / opacity
   float4 *box;   // conservative pixel-centre box of the contributing ellipse
   float4 *q;     // conic_a, conic_b, conic_c, qlim = min(9, 2 ln(255 o)) for the block test
 };
@@ -101,7 +101,7 @@ __device__ __forceinline__ void stage_from(const float4 r0, const float4 r1, con
   s.a[j] = make_float4(r0.x, r0.y, __fmul_rn(kExpScale, ca), __fmul_rn(2.f * kExpScale, cb));
   s.b[j] = make_float4(__fmul_rn(kExpScale, cc), -o, r2.x, r2.y);
   const float pcut = fmaxf(9.f * kExpScale, -__log2f(255.f * o));
-  s.c[j] = make_float4(r2.z, __uint_as_float(pid), pcut, 0.f);
+  s.c[j] = make_float4(r2.z, __uint_as_float(pid), pcut, __fdividef(-1.f, o));   // (read only where the splat blends: o >= 1/255)
   const float qlim = fminf(kQMax, 2.f * __logf(255.f * o));
   s.q[j] = make_float4(ca, cb, cc, qlim);
   const float detq = ca * cc - cb * cb;

@@ -59,7 +59,7 @@ __device__ __forceinline__ void warp_reduce_9(const float (&v)[9], int lane, flo
 // Per-splat sums of a thread's pixels, kept as two packed lanes (the two
 // pixels of a pair) and added lane to lane once per splat.
 struct AdjSums {
-  f32x2 a5, a6, a7, a8, q1, qy, qyy;
+  f32x2 a6, a7, a8, q1, qy, qyy;
 };
 
 // Two pixels' shares of the adjoint of a blended splat, pixels h and h + 1
@@ -68,17 +68,19 @@ struct AdjSums {
 // skipped this splat in the forward and passes its footprint test.  Per pixel, T
 // (transmittance after the splat) becomes T before it; GS = dL/dC . S, S
 // being the colour composited behind (background included), takes the
-// splat's own term (only that dot product enters dL/dalpha); the colour and
-// opacity gradients go to the sums a5..a8.  The conic and mean gradients
-// are linear in dq = dL/dq, so a pixel only adds dq, dq dy and dq dy^2 to
-// q1, qy, qyy (dx is common to a thread's pixels) and the caller forms them
-// once per splat.  A pixel that skips the splat (ok false: outside the
-// footprint, or past its last blended entry) takes alpha 0, which leaves
-// its T and GS unchanged and adds 0 to every sum, so the pair runs without
-// a branch.  GS is kept negated (NGS = -dL/dC . S) and alpha as nal =
-// -alpha (the staged opacity is negated), which turns dL/dalpha into one
-// fused multiply-add.  kFirst: this pair starts the sums instead of adding
-// to them.
+// splat's own term (only that dot product enters dL/dalpha); the colour gradients go
+// to the sums a6..a8.  The conic, mean and opacity gradients are linear in
+// dq = 2 dL/dq = -alpha dL/dalpha (alpha = o 2^power, power = k q, unclamped
+// pixels only): a pixel adds dq, dq dy and dq dy^2 to q1, qy, qyy (dx
+// is common to a thread's pixels) and the caller forms them once per
+// splat, dL/do being -sum dq / o.  A pixel that skips the splat (ok false:
+// outside the footprint, or past its last blended entry) takes alpha 0,
+// which leaves its T and GS unchanged and adds 0 to every sum, so the pair
+// runs without a branch: its exponent is replaced, which makes 2^power and
+// all that follows from it 0 with no further select.  GS is kept negated
+// (NGS = -dL/dC . S) and alpha as nal = -alpha (the staged opacity is
+// negated), which turns dL/dalpha into one fused multiply-add.  kFirst: this
+// pair starts the sums instead of adding to them.
 template <bool kFirst>
 __device__ __forceinline__ void pixel_adjoint2(const float4 &a, const float4 &b, const float4 &c4, f32x2 pw, f32x2 dy,
                                                bool ok0, bool ok1, f32x2 g0, f32x2 g1, f32x2 g2, float &T0,
@@ -87,14 +89,12 @@ __device__ __forceinline__ void pixel_adjoint2(const float4 &a, const float4 &b,
   unpack2(pw, p0, p1);
   // power <= 0 for the positive-definite conics of pk_project_and_sh: G in
   // [0, 1] at every pixel, and a skipping pixel's zero alpha zeroes its terms
-  const float G0 = ex2_approx(p0), G1 = ex2_approx(p1);
+  const float G0 = ex2_approx(ok0 ? p0 : -1e30f), G1 = ex2_approx(ok1 ? p1 : -1e30f);
   // 1 + nal, nal Ti and the sums below are exactly the negations of the
   // alpha forms
   float r0, r1;
   unpack2(mul2(dup2(b.y), pack2(G0, G1)), r0, r1);
-  const bool cl0 = r0 < -kAlphaMax, cl1 = r1 < -kAlphaMax;
-  const float nal0 = ok0 ? (cl0 ? -kAlphaMax : r0) : 0.f;
-  const float nal1 = ok1 ? (cl1 ? -kAlphaMax : r1) : 0.f;
+  const float nal0 = fmaxf(r0, -kAlphaMax), nal1 = fmaxf(r1, -kAlphaMax);
   const f32x2 nal = pack2(nal0, nal1);
   float om0, om1;
   unpack2(add2(dup2(1.f), nal), om0, om1);
@@ -107,8 +107,7 @@ __device__ __forceinline__ void pixel_adjoint2(const float4 &a, const float4 &b,
   // dL/dalpha = (T g.rgb - g.S) / (1 - alpha), with NGS = -g.S
   const f32x2 gr = fma2(g2, dup2(c4.x), fma2(g1, dup2(b.w), mul2(g0, dup2(b.z))));
   const f32x2 NGSv = pack2(NGS0, NGS1);
-  float da0, da1;
-  unpack2(mul2(fma2(Tv, gr, NGSv), inv), da0, da1);
+  const f32x2 da = mul2(fma2(Tv, gr, NGSv), inv);
   unpack2(fma2(nwT, gr, NGSv), NGS0, NGS1);
   // a skipping pixel has alpha 0: 1 / (1 - 0) = 1 exactly, T stays
   T0 = ti0;
@@ -117,10 +116,8 @@ __device__ __forceinline__ void pixel_adjoint2(const float4 &a, const float4 &b,
   s.a6 = kFirst ? mul2(nwT, g0) : fma2(nwT, g0, s.a6);
   s.a7 = kFirst ? mul2(nwT, g1) : fma2(nwT, g1, s.a7);
   s.a8 = kFirst ? mul2(nwT, g2) : fma2(nwT, g2, s.a8);
-  // alpha = o 2^power, power = k q: dL/dq = -alpha dL/dalpha / 2 (unclamped pixels only)
-  const f32x2 dav = pack2(ok0 && !cl0 ? da0 : 0.f, ok1 && !cl1 ? da1 : 0.f);
-  s.a5 = kFirst ? mul2(dav, pack2(G0, G1)) : fma2(dav, pack2(G0, G1), s.a5);
-  const f32x2 dq = mul2(mul2(dup2(0.5f), nal), dav);
+  // a clamped alpha does not depend on the exponent
+  const f32x2 dq = mul2(pack2(r0 < -kAlphaMax ? 0.f : r0, r1 < -kAlphaMax ? 0.f : r1), da);
   const f32x2 t = mul2(dq, dy);
   s.q1 = kFirst ? dq : add2(s.q1, dq);
   s.qy = kFirst ? t : add2(s.qy, t);
@@ -133,17 +130,23 @@ __device__ __forceinline__ float lane_sum(f32x2 v) {
   return lo + hi;
 }
 
-// Conic and mean gradients of a splat from the pixel sums q1 = sum dq,
-// qy = sum dq dy, qyy = sum dq dy^2 (common dx): d/dconic = dq (dx^2,
-// 2 dx dy, dy^2), dq/dm = -2 conic d = -(2 A dx + B dy, B dx + 2 C dy) / k.
-__device__ __forceinline__ void conic_mean_grads(const float4 &a, const float4 &b, float dx, float q1, float qy,
-                                                 float qyy, float (&acc)[9]) {
-  const float dq1 = dx * q1;
-  acc[2] = dx * dq1;
-  acc[3] = 2.f * dx * qy;
+// Conic, mean and opacity gradients of a splat from the pixel sums q1 =
+// sum dq, qy = sum dq dy, qyy = sum dq dy^2 (common dx; dq as above): with
+// dL/dq = dq / 2, d/dconic = dL/dq (dx^2, 2 dx dy, dy^2), dq/dm = -2 conic d =
+// -(2 A dx + B dy, B dx + 2 C dy) / k, each up to the constant factor that
+// grad_factor gives the lane that holds the complete sum.
+__device__ __forceinline__ void conic_mean_grads(const float4 &a, const float4 &b, float nio, float dx, float q1,
+                                                 float qy, float qyy, float (&acc)[9]) {
+  const float qx = dx * q1, hb = 0.5f * a.w;
+  acc[0] = fmaf(a.z, qx, hb * qy);
+  acc[1] = fmaf(hb, qx, b.x * qy);
+  acc[2] = dx * qx;
+  acc[3] = dx * qy;
   acc[4] = qyy;
-  acc[0] = -kInvExpScale * (2.f * a.z * dq1 + a.w * qy);
-  acc[1] = -kInvExpScale * (a.w * dq1 + 2.f * b.x * qy);
+  acc[5] = nio * q1;   // sum dL/dalpha 2^power = -q1 / o
+}
+__device__ __forceinline__ float grad_factor(int idx) {
+  return idx < 2 ? -kInvExpScale : idx == 2 || idx == 4 ? 0.5f : idx < 6 ? 1.f : -1.f;   // colours: -alpha T dL/dC
 }
 
 // kTma: the records of the next (earlier) batch are fetched into shared
@@ -177,6 +180,7 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
   // the lane that adds each of the nine sums: lanes 0, 4, ..., 28 the
   // scattered eight, lane 1 the ninth (-1: none)
   const int my_idx = (lane & 3) == 0 ? reduce_scatter8_index(lane) : (lane == 1 ? 8 : -1);
+  const float my_factor = grad_factor(my_idx);
   uint32_t evals = 0;   // per thread: far below 2^32
   uint32_t phase = 0;
   bool timed_out = false;
@@ -372,14 +376,14 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
           }
           {
             float acc[9];
-            acc[5] = lane_sum(sums.a5);
-            acc[6] = -lane_sum(sums.a6);   // the colour sums hold -alpha T dL/dC
-            acc[7] = -lane_sum(sums.a7);
-            acc[8] = -lane_sum(sums.a8);
-            conic_mean_grads(a, b, dx, lane_sum(sums.q1), lane_sum(sums.qy), lane_sum(sums.qyy), acc);
+            acc[6] = lane_sum(sums.a6);
+            acc[7] = lane_sum(sums.a7);
+            acc[8] = lane_sum(sums.a8);
+            conic_mean_grads(a, b, c4.w, dx, lane_sum(sums.q1), lane_sum(sums.qy), lane_sum(sums.qyy), acc);
             float s8, s9;
             warp_reduce_9(acc, lane, s8, s9);
-            if (my_idx >= 0) atomicAdd(grad2d + (size_t)__float_as_uint(c4.y) * kG2d + my_idx, lane == 1 ? s9 : s8);
+            if (my_idx >= 0)
+              atomicAdd(grad2d + (size_t)__float_as_uint(c4.y) * kG2d + my_idx, my_factor * (lane == 1 ? s9 : s8));
           }
         }
       }
