@@ -1298,8 +1298,9 @@ pk_status radix_pass_rb(const uint32_t *kin, const uint32_t *vin, uint32_t *kout
                         DigitBase dbase, uint64_t *csum, pk_device_status *status, SegSpec sp, uint32_t *abort_flag,
                         uint32_t first_polls, bool try_single, const Unpack &up, cudaStream_t st) {
   using C = Radix<RB, IT>;
-  if (cudaFuncSetAttribute(k_radix_downsweep<RB, IT, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)Down<RB, IT>::kSmem) != cudaSuccess)
+  static KernelInfo info;
+  const auto downsweep = k_radix_downsweep<RB, IT, kMode>;
+  if (resident_ctas(info, reinterpret_cast<const void *>(downsweep), kThreads, Down<RB, IT>::kSmem) == 0)
     return PK_ERR_CUDA;
   const uint32_t mask = (1u << bits) - 1u;
   if (dbase != kSolo)
@@ -1345,13 +1346,6 @@ pk_status radix_pass(bool entries, int rb, const uint32_t *kin, const uint32_t *
   if (rb > 8) PK_PASS(11, kPairItems, 0);
   PK_PASS(8, kPairItems, 0);
 #undef PK_PASS
-}
-
-int sm_count() {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return std::max(1, sms);
 }
 
 // Blocks of an unsegmented pass over at most `items` pairs or entries, or
@@ -1469,9 +1463,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   uint32_t *dv = at<uint32_t>(ws, L.dval);
   const uint64_t *n_valid = &ctr->n_valid;
   const uint64_t pairs = (uint64_t)p->pairs;
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   // segmented sorts (V >= 2): the depth passes sort each view's pairs in
   // place, the tile passes each view's entries on per-view local tile ids
   int4 tab_host[2 * kSortBlocks];
@@ -1536,7 +1528,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   np = radix_plan(key_bits, rt, widths);
   uint32_t *vbuf[2] = {(np & 1) ? dv : sorted_vals, (np & 1) ? sorted_vals : dv};
   uint32_t *kbuf[2] = {dk0, dk1};
-  k_emit<<<std::max(1, sms) * 32, kThreads, 0, st>>>(records, pval, offs, pinfo, ctr, views, p->N, p->pairs, p->T,
+  k_emit<<<sms * 32, kThreads, 0, st>>>(records, pval, offs, pinfo, ctr, views, p->N, p->pairs, p->T,
                                                       p->opts.bin_mode, seg ? key_bits : 0, packed ? pbits : 0,
                                                       kbuf[0], vbuf[0], status);
   // Digits from the top down: each tile's entries still end up contiguous
@@ -1562,9 +1554,9 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
     if (e != PK_OK) return e;
   }
   if (packed)
-    k_range_fix<<<std::max(1, sms) * 4, kThreads, 0, st>>>(tile_ranges, (uint32_t)p->n_tiles, ctr);
+    k_range_fix<<<sms * 4, kThreads, 0, st>>>(tile_ranges, (uint32_t)p->n_tiles, ctr);
   else
-    k_ranges<<<std::max(1, sms) * 16, kThreads, 0, st>>>(kbuf[np & 1], seg ? key_bits : 0,
+    k_ranges<<<sms * 16, kThreads, 0, st>>>(kbuf[np & 1], seg ? key_bits : 0,
                                                           at<uint32_t>(ws, L.toff), ctr, tile_ranges, p->V,
                                                           (uint32_t)p->n_tiles, status);
   return check_launch();

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <atomic>
 #include <initializer_list>
 #include <utility>
 
@@ -108,6 +109,16 @@ __host__ __device__ inline T *at(void *base, size_t off) {
 // Host-side launch helpers (implemented in pk_plan.cu).
 pk_status check_launch();
 bool aligned16(const void *p);
+// SMs of the current device (at least 1), looked up once per device.
+int sm_count();
+// Resident CTAs per SM (at least 1) of a kernel on the current device, with
+// its dynamic shared memory allowed; looked up once per device and kernel
+// (`info`: a static of the launching code, one per kernel), since the two
+// driver calls cost more host time than a launch.  0: the device refuses it.
+struct KernelInfo {
+  std::atomic<int> per_sm[64]{};
+};
+int resident_ctas(KernelInfo &info, const void *kernel, int threads, size_t smem);
 // Zero up to four (pointer, bytes) ranges with one kernel (4-byte aligned
 // pointers, sizes multiples of 4 bytes).
 pk_status zero_async(std::initializer_list<std::pair<void *, size_t>> spans, cudaStream_t st);

@@ -60,6 +60,30 @@ __global__ void k_status_out(const uint32_t *__restrict__ st, int nst, const uin
 // One kernel instead of cudaMemsetAsync: inside a CUDA graph a memset node
 // may be run by a copy engine, where it queues behind (and is delayed by)
 // unrelated host <-> device copies of other streams.
+int sm_count() {
+  static std::atomic<int> cached[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  const bool keep = dev >= 0 && dev < 64;
+  int n = keep ? cached[dev].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+  if (keep) cached[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
+
+int resident_ctas(KernelInfo &info, const void *kernel, int threads, size_t smem) {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const bool keep = dev >= 0 && dev < 64;
+  if (keep && (n = info.per_sm[dev].load(std::memory_order_acquire)) > 0) return n;
+  if (smem > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    return 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess || n < 1) n = 1;
+  if (keep) info.per_sm[dev].store(n, std::memory_order_release);
+  return n;
+}
+
 pk_status zero_async(std::initializer_list<std::pair<void *, size_t>> spans, cudaStream_t st) {
   ZeroSpans z{};
   uint64_t most = 0;

@@ -409,13 +409,10 @@ pk_status launch_bwd(const pk_plan *p, const float *records, const uint32_t *sor
                      const uint64_t *tile_ranges, const float *T_final, const uint32_t *n_contrib,
                      const float *dL_dimage, float *grad2d, void *ws, DevCounters *ctr, pk_device_status *status,
                      cudaStream_t st) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_bwd<kBatch, kBwdTma, kBwdPx, kT, kCount>,
-                                                Geo<kBwdPx>::kThreads, 0);
-  if (sms < 1) sms = 1;
-  if (per_sm < 1) per_sm = 1;
+  static KernelInfo info;
+  const int sms = sm_count();
+  const auto kernel = k_raster_bwd<kBatch, kBwdTma, kBwdPx, kT, kCount>;
+  const int per_sm = std::max(1, resident_ctas(info, reinterpret_cast<const void *>(kernel), Geo<kBwdPx>::kThreads, 0));
   const int64_t items = p->n_tiles * (kT / kTileSide) * (kT / kTileSide);
   int64_t grid = (int64_t)sms * per_sm;
   if (grid > items) grid = items;

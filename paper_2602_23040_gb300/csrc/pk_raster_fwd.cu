@@ -289,13 +289,10 @@ pk_status launch_fwd(const pk_plan *p, const float *records, const uint32_t *sor
                      const uint64_t *tile_ranges, float *image, float *T_final, uint32_t *n_contrib, void *ws,
                      DevCounters *ctr, pk_device_status *status, const float *target, float *dimg, float *clear,
                      uint64_t clear_floats, cudaStream_t st) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_raster_fwd<kBatch, kFwdTma, kFwdPx, kT, kCount>,
-                                                Geo<kFwdPx>::kThreads, 0);
-  if (sms < 1) sms = 1;
-  if (per_sm < 1) per_sm = 1;
+  static KernelInfo info;
+  const int sms = sm_count();
+  const auto kernel = k_raster_fwd<kBatch, kFwdTma, kFwdPx, kT, kCount>;
+  const int per_sm = std::max(1, resident_ctas(info, reinterpret_cast<const void *>(kernel), Geo<kFwdPx>::kThreads, 0));
   const int64_t items = p->n_tiles * (kT / kTileSide) * (kT / kTileSide);
   int64_t grid = (int64_t)sms * per_sm;
   if (grid > items) grid = items;
