@@ -208,9 +208,9 @@ def measured_fp32_per_eval(stage):
 
 
 def launches_per_step(plan):
-    # gather 2, project 1, bin_and_sort (as the library counts it), fwd with the loss 2 (zeroing +
-    # compositing), bwd 2 (zeroing + adjoint), scatter 1
-    return 2 + 1 + int(plan.sizes.bin_kernels) + 5
+    # gather 2, project 1, bin_and_sort (as the library counts it), fwd with the loss 3 (zeroing +
+    # compositing + long lists), bwd 4 (zeroing + adjoint + long lists' sums and segments), scatter 1
+    return 2 + 1 + int(plan.sizes.bin_kernels) + 8
 
 
 # ---------------------------------------------------------------------------

@@ -35,6 +35,12 @@ constexpr int kSortBlocks = 2560;     // most radix blocks of one pass (histogra
 constexpr int kMaxRadixBits = 11;     // widest radix digit (pk_options.sort_bits_*: 8 or 11)
 constexpr uint64_t kMaxEntries = uint64_t(1) << 35;   // most (pair, tile) entries of a plan
 
+// Long lists (pk_raster.cuh): most of a pass, and most segments of the
+// backward's in a pass.
+constexpr uint32_t kLongMaxItems = 1024;
+constexpr uint32_t kSplitMaxUnits = 24576;
+constexpr uint32_t kSplitBlock = 256;   // pixels of a 16 x 16 block
+
 // Per-view constants on the device, 144 bytes.
 struct alignas(16) DevView {
   float R[9];
@@ -51,11 +57,19 @@ struct alignas(16) DevView {
 };
 static_assert(sizeof(DevView) % 16 == 0, "DevView layout");
 
+// Work counters of one compositing pass: the tile queue of its persistent
+// kernel, its CTAs that have ended, and the long lists (pk_raster.cuh): items
+// and (backward) units handed out, most segments of an item, and the queues
+// of the kernels that follow.
+struct RasterQueue {
+  uint32_t tile, exited, items, units, max_seg, seg_q[2], pad;
+};
+
 // Internal device scalars kept after the public status block.
 struct DevCounters {
   uint64_t n_valid;        // pairs with >= 1 tile (after the compaction scan)
   uint64_t dups;           // entries emitted (0 on overflow); 64-bit, as are entry positions
-  uint32_t tile_queue[4];  // persistent-kernel work counters
+  RasterQueue raster[2];   // the forward's and the backward's
   uint64_t scan_total;     // total of the last scan
   double loss_acc;         // sum of |image - target| of the last loss call
   double ssim_acc;         // sum of the SSIM map of the last photometric loss call
@@ -75,6 +89,7 @@ struct WsLayout {
   int sort_cap;            // most radix blocks of one pass (counters in hist)
   size_t mask_tmp;         // one motion mask's worth of words (dilation scratch)
   size_t mask_coarse;      // per view, one bit per 32 x 32-pixel block: any moving pixel
+  size_t longs, split;     // the forward's long lists and the backward's split lists (pk_raster.cuh)
   size_t total;
 };
 
@@ -90,6 +105,7 @@ struct pk_plan {
   int32_t tile_bits;       // bits needed for a global tile id
   int32_t num_sms;
   uint32_t first_polls;    // polls of the first bounded wait on a bulk-copied batch
+  uint32_t long_items, split_units;   // long lists (forward) and segments of split ones that the workspace holds
   pk::WsLayout ws;
   pk::DevView *h_views;    // host copies uploaded by pk_workspace_init
   uint32_t *h_toff;        // [V+1] tile offsets (global tile id -> view)

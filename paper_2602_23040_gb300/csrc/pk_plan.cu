@@ -6,7 +6,7 @@
 
 #include <new>
 
-#include "pk_common.cuh"
+#include "pk_raster.cuh"
 #include "pk_tma.cuh"
 
 using namespace pk;
@@ -355,6 +355,13 @@ extern "C" pk_status pk_plan_create(const pk_atlas_desc *desc, const pk_view *vi
   L.vseg = take(sizeof(uint64_t) * 2 * (V + 1));
   L.mask_tmp = take(sizeof(uint32_t) * (size_t)p->mask_words);
   L.mask_coarse = take(sizeof(uint32_t) * (size_t)p->coarse_words);
+  // long lists (at most one per work item, and per CTA of the last few) and segments of
+  // split ones (64 entries at least, four quadrants' lists per tile)
+  const uint64_t blocks16 = (uint64_t)p->n_tiles * (o.tile / kTileSide) * (o.tile / kTileSide);
+  p->long_items = (uint32_t)std::min<uint64_t>(kLongMaxItems, blocks16);
+  L.longs = take(LongItems::bytes(p->long_items));
+  p->split_units = (uint32_t)std::min<uint64_t>(kSplitMaxUnits, 4 * maxd / 64 + 1);
+  L.split = take(SplitBwd::bytes(p->long_items, p->split_units));
   L.total = off;
   *out = p;
   return PK_OK;

@@ -193,4 +193,142 @@ __device__ __forceinline__ bool block_may_hit(const float4 &box, const float4 &q
   return best <= q.w * 1.001f + 1e-3f;
 }
 
+// ---------------------------------------------------------------------------
+// Long lists.  One CTA walks its block's list in order, so a long list of a
+// block that does not saturate (the rim of a dense cluster, a small view of
+// many splats) is a serial chain of some 40 ns per entry on one CTA while the
+// rest of the GPU has run dry: a 97 x 403 view of 34 K splats kept the
+// forward and the backward for 1.5 and 2.0 ms, most of it one CTA.
+//
+// So once few CTAs are left of a pass of not too many work items, one that
+// still has a long way to go in its list leaves the rest of it to kernels
+// that spread one list over more of the GPU (k_raster_fwd_long, the backward's
+// segments below).  While more of them run, lists are walked whole, which
+// takes less work in all: the forward's other kernel spends about 2.4 times
+// the instructions per entry, the backward's 1.4 times.  The lines lie at an eighth and a quarter of the resident CTAs:
+// with the hand-over as soon as the tile queue is dry instead, 44 views of
+// 195 x 195 pixels on 253 K splats take 11.1 ms for 6.7 (whole lists: 9.2).
+// And passes of more than kLongPasses work items per resident CTA run
+// without it: their tail is short, and the test in its loop costs the
+// forward 2 % (52-view rig, 306 K items: 4.11 -> 4.20 ms; at 66 K items a
+// 16-view step gains 13 %).
+constexpr int64_t kLongPasses = 100;
+__device__ __forceinline__ bool few_left(const RasterQueue *q, uint32_t few) {
+  return gridDim.x - *reinterpret_cast<const volatile uint32_t *>(&q->exited) <= few;
+}
+// Entries walked and left: a hand-over costs about as much as 256; where there
+// are many more work items than CTAs the last ones end at about the same
+// time, and only a walk of 1,024 more is worth one.
+__device__ __forceinline__ uint32_t long_least(uint32_t n_items) {
+  return n_items <= 4u * gridDim.x ? 256u : 1024u;
+}
+// A launch that leaves most of the GPU idle from its start: lists of kTinyList
+// entries and more go over before their first batch.
+constexpr uint32_t kTinyList = 128;
+
+// What the forward hands over: work item, entries walked (a multiple of every
+// batch) and, per pixel (row-major in the block), colour sum and
+// transmittance, and the last blended entry (bit 31: the pixel has stopped).
+// w = kNoPair: a slot taken for a block that ended by itself.
+struct LongItems {
+  float4 *state;
+  uint32_t *last, *w, *first;
+  static size_t bytes(uint64_t slots) { return slots * (kSplitBlock * (sizeof(float4) + sizeof(uint32_t)) + 8); }
+  static LongItems of(void *base, uint64_t slots) {
+    LongItems l;
+    l.state = static_cast<float4 *>(base);
+    l.last = reinterpret_cast<uint32_t *>(l.state + slots * kSplitBlock);
+    l.w = l.last + slots * kSplitBlock;
+    l.first = l.w + slots;
+    return l;
+  }
+};
+
+// The backward's split lists: the rest of a long walk is cut into segments
+// that other CTAs walk at the same time.  A segment's transmittance and
+// colour behind follow from the later segments' products of (1 - alpha) and
+// colour sums (compositing is associative), which a first pass over the
+// segments takes.  (The forward keeps one rounding order whatever a list
+// holds besides a pixel's contributors, so it does not cut its lists.)
+// Segments of split_least entries at least (one batch; half a batch in a
+// launch that leaves most of the GPU idle from its start), 64 of the first 128
+// lists at most and 16 of the others, so that a pass's segments fill the GPU a
+// few times over; all of about the same length, since the longest is the
+// pass's time.
+__device__ __forceinline__ uint32_t split_least(uint32_t few) { return gridDim.x <= few ? 64u : 128u; }
+__device__ __forceinline__ uint32_t split_segments(uint32_t len, uint32_t least, uint32_t item) {
+  return min(len / least, item < 128u ? 64u : 16u);
+}
+
+// A split list: work item w (tile and quadrant), its first unit (segment
+// slot), segments of x entries (the last the rest of them), entries.
+struct SplitItem {
+  uint32_t w, unit0, nseg, x, len;
+};
+
+// Per unit and pixel of the block (row-major): tl = product of (1 - alpha)
+// over the segment, ls = sum of alpha T dL/dC.rgb with T = 1 before it.  Per
+// item and pixel: T and -dL/dC.(colour behind) at the end of its entries.
+struct SplitBwd {
+  float2 *state;
+  float *tl, *ls;
+  SplitItem *items;
+  static size_t bytes(uint64_t items, uint64_t units) {
+    return items * (sizeof(SplitItem) + kSplitBlock * sizeof(float2)) + units * kSplitBlock * 2 * sizeof(float);
+  }
+  static SplitBwd of(void *base, uint64_t items, uint64_t units) {
+    SplitBwd s;
+    s.state = static_cast<float2 *>(base);
+    s.tl = reinterpret_cast<float *>(s.state + items * kSplitBlock);
+    s.ls = s.tl + units * kSplitBlock;
+    s.items = reinterpret_cast<SplitItem *>(s.ls + units * kSplitBlock);
+    return s;
+  }
+};
+
+// Enter the first `len` entries of a list as a split item; its index, or
+// kNoPair when the slots are used up (the caller then walks on).  One thread.
+__device__ __forceinline__ uint32_t split_enter(RasterQueue *q, SplitItem *items, uint32_t max_items, uint32_t units,
+                                                uint32_t w, uint32_t len, uint32_t least) {
+  const uint32_t i = atomicAdd(&q->items, 1u);
+  if (i >= max_items) return kNoPair;
+  const uint32_t n = split_segments(len, least, i), x = (len + n - 1u) / n, nseg = (len + x - 1u) / x;
+  const uint32_t unit0 = atomicAdd(&q->units, nseg);
+  const bool fits = unit0 < units && nseg <= units - unit0;
+  items[i] = SplitItem{w, unit0, fits ? nseg : 0u, x, len};
+  if (!fits) return kNoPair;
+  atomicMax(&q->max_seg, nseg);
+  return i;
+}
+
+// The next (item, segment) of queue k, segment `first` or later.  False when
+// none is left.  One thread.
+__device__ __forceinline__ bool split_next(RasterQueue *q, const SplitItem *items, uint32_t max_items, int k,
+                                           uint32_t first, uint32_t &it, uint32_t &seg) {
+  const uint32_t n = min(q->items, max_items), most = q->max_seg;
+  if (n == 0 || most <= first) return false;
+  const uint64_t total = (uint64_t)n * (most - first);
+  for (;;) {
+    const uint32_t v = atomicAdd(&q->seg_q[k], 1u);
+    if (v >= total) return false;
+    seg = first + v / n;
+    it = v % n;
+    if (seg < items[it].nseg) return true;
+  }
+}
+
+// Bounds of a warp's pixel centres that satisfy `on` (any of the warp's
+// pixels; the empty rectangle otherwise).
+struct WarpRect {
+  float x0, x1, y0, y1;
+};
+__device__ __forceinline__ WarpRect warp_rect(bool any, int x, int ylo, int yhi) {
+  WarpRect r;
+  r.x0 = (float)__reduce_min_sync(0xffffffffu, any ? x : 0x3fffffff) + 0.5f;
+  r.x1 = (float)__reduce_max_sync(0xffffffffu, any ? x : -0x3fffffff) + 0.5f;
+  r.y0 = (float)__reduce_min_sync(0xffffffffu, any ? ylo : 0x3fffffff) + 0.5f;
+  r.y1 = (float)__reduce_max_sync(0xffffffffu, any ? yhi : -0x3fffffff) + 0.5f;
+  return r;
+}
+
 }  // namespace pk

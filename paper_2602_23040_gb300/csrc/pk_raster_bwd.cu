@@ -157,20 +157,29 @@ __device__ __forceinline__ float grad_factor(int idx) {
 // kT: side of the tiles the lists were binned for; each CTA takes a 16 x 16
 // quadrant of one, as in the forward.  kCount: count the evaluations (a
 // measurement; the variant without it carries no counter in its loop).
-template <int kBatch, bool kTma, int kPx, int kT, bool kCount>
+// kSplit: kEnter, long walks go to the split lists once at most `few` CTAs are
+// left; kSegments, the work items are the segments of those, which k_bwd_sums
+// summed; a segment's transmittance and colour behind follow from the state
+// at the end of its item's entries and the later segments' sums.
+enum BwdSplit { kNoSplit, kEnter, kSegments };
+
+template <int kBatch, bool kTma, int kPx, int kT, bool kCount, BwdSplit kSplit>
 __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_raster_bwd(
     const float *__restrict__ rec, const uint32_t *__restrict__ vals, const uint64_t *__restrict__ ranges,
     const DevView *__restrict__ views, const uint32_t *__restrict__ toff, int V, uint32_t n_items, float bg0,
     float bg1, float bg2, const float *__restrict__ Tfin, const uint32_t *__restrict__ ncontrib,
-    const float *__restrict__ dimg, float *__restrict__ grad2d, uint32_t *queue, unsigned long long *evals_out,
-    pk_device_status *status, uint32_t first_polls, uint32_t npairs) {
+    const float *__restrict__ dimg, float *__restrict__ grad2d, unsigned long long *evals_out,
+    pk_device_status *status, uint32_t first_polls, uint32_t npairs, SplitBwd split, uint32_t split_items,
+    uint32_t split_units, RasterQueue *rq, uint32_t few) {
+  constexpr bool kSegs = kSplit == kSegments;
+  static_assert(!kSegs || (!kTma && !kCount), "split segments are staged by plain loads and not counted");
   using G = Geo<kPx>;
   constexpr uint32_t kQuads = (kT / kTileSide) * (kT / kTileSide);   // CTAs per list tile
   __shared__ float4 s_a[kBatch], s_b[kBatch], s_c[kBatch], s_box[kBatch], s_q[kBatch];
   __shared__ __align__(16) float4 s_raw[kTma ? 3 * kBatch : 1];
   __shared__ uint32_t s_pid[kTma ? kBatch : 1];
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ uint32_t s_tile;
+  __shared__ uint32_t s_tile, s_unit, s_seg;
   __shared__ int s_view;
   __shared__ uint32_t s_wmax[G::kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -202,9 +211,16 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
     }
   };
   for (;;) {
-    // work item: (list tile t, 16 x 16 quadrant q of it)
+    // work item: (list tile t, 16 x 16 quadrant q of it), or a segment of a split one
     if (tid == 0) {
-      const uint32_t w = atomicAdd(queue, 1u);
+      uint32_t w = n_items, it, seg;
+      if (!kSegs) {
+        w = atomicAdd(&rq->tile, 1u);
+      } else if (split_next(rq, split.items, split_items, 1, 0u, it, seg)) {
+        s_unit = it;
+        s_seg = seg;
+        w = split.items[it].w;
+      }
       s_tile = w;
       s_view = w < n_items ? view_of_tile(toff, V, w / kQuads) : -1;
     }
@@ -254,6 +270,23 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
       }
       // -dL/dC . (colour composited behind the current splat, background included)
       NGS[q] = -(T[q] * fmaf(g2[q], bg2, fmaf(g1[q], bg1, g0[q] * bg0)));
+      if (kSegs) {
+        // from the item's end through the segments behind this one: T before
+        // a segment is T after it over its product, the colour behind grows
+        // by its sum
+        const SplitItem &it = split.items[s_unit];
+        const size_t px = (oy + q * G::kRowStep) * kTileSide + ox, pu = (size_t)it.unit0 * kSplitBlock + px;
+        const float2 end = split.state[(size_t)s_unit * kSplitBlock + px];
+        T[q] = end.x;
+        NGS[q] = end.y;
+        nc[q] = min(nc[q], it.len);
+        for (uint32_t j = it.nseg - 1; j > s_seg; --j) {
+          const float Tb = __fdividef(T[q], split.tl[pu + (size_t)j * kSplitBlock]);
+          NGS[q] = fmaf(-Tb, split.ls[pu + (size_t)j * kSplitBlock], NGS[q]);
+          T[q] = Tb;
+        }
+        if (s_seg + 1 < it.nseg) nc[q] = min(nc[q], (s_seg + 1) * it.x);
+      }
       ncmax = max(ncmax, nc[q]);
     }
     const uint32_t wmax = __reduce_max_sync(0xffffffffu, ncmax);
@@ -262,6 +295,11 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
     uint32_t tmax = 0;
 #pragma unroll
     for (int w = 0; w < G::kWarps; ++w) tmax = max(tmax, s_wmax[w]);
+    uint32_t lo = 0;   // first list position of this walk
+    if (kSegs) {
+      lo = s_seg * split.items[s_unit].x;
+      if (tmax <= lo) tmax = lo;
+    }
     if (kTma && tmax > 0) {
       const uint32_t b0 = tmax > (uint32_t)kBatch ? tmax - kBatch : 0u;
       if (tid == 0) mbar_expect_tx(&s_bar, (tmax - b0) * 3u * (uint32_t)sizeof(float4));
@@ -274,16 +312,39 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
     constexpr int kPer = (kBatch + G::kThreads - 1) / G::kThreads;
     uint32_t npid[kPer];
     if (!kTma) {
-      const uint32_t b0 = tmax > (uint32_t)kBatch ? tmax - kBatch : 0u;
+      const uint32_t b0 = tmax - lo > (uint32_t)kBatch ? tmax - kBatch : lo;
 #pragma unroll
       for (int u = 0; u < kPer; ++u) {
         const int j = tid + u * G::kThreads;
         npid[u] = j < kBatch && b0 + (uint32_t)j < tmax ? __ldg(vals + s + b0 + j) : 0u;
       }
     }
-    for (uint32_t end = tmax; end > 0;) {
-      const uint32_t beg = end > (uint32_t)kBatch ? end - kBatch : 0u;
+    for (uint32_t end = tmax; end > lo;) {
+      const uint32_t beg = end - lo > (uint32_t)kBatch ? end - kBatch : lo;
       const int nb = (int)(end - beg);
+      // a long walk of one of the last CTAs: the entries left go to the split lists
+      if (kSplit == kEnter && end >= (n_items <= 4u * gridDim.x ? 2u * split_least(few) : 2u * long_least(n_items))) {
+        if (tid == 0)
+          s_unit = few_left(rq, few)
+                       ? split_enter(rq, split.items, split_items, split_units, w, end, split_least(few))
+                       : kNoPair;
+        __syncthreads();
+        const uint32_t it = s_unit;
+        if (it != kNoPair) {
+#pragma unroll
+          for (int q = 0; q < kPx; ++q)
+            split.state[(size_t)it * kSplitBlock + (oy + q * G::kRowStep) * kTileSide + ox] = make_float2(T[q], NGS[q]);
+          if (kTma) {   // this batch's copies land before the block goes on
+            if (!mbar_wait_bounded(&s_bar, phase, first_polls)) {
+              timed_out = true;
+              mbar_wait_bounded(&s_bar, phase);
+            }
+            phase ^= 1u;
+            timed_out = __syncthreads_or(timed_out);
+          }
+          break;
+        }
+      }
       if (kTma) {
         if (!mbar_wait_bounded(&s_bar, phase, first_polls)) {
           timed_out = true;
@@ -316,7 +377,7 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
           const int j = tid + u * G::kThreads;
           if (j < nb) stage_splat(rec, npid[u], npairs, st, j, status);
         }
-        const uint32_t nbeg = beg > (uint32_t)kBatch ? beg - kBatch : 0u;
+        const uint32_t nbeg = beg - lo > (uint32_t)kBatch ? beg - kBatch : lo;
 #pragma unroll
         for (int u = 0; u < kPer; ++u) {
           const int j = tid + u * G::kThreads;
@@ -395,6 +456,7 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
     }
     __syncthreads();
   }
+  if (kSplit == kEnter && tid == 0) atomicAdd(&rq->exited, 1u);
   if (kCount) {
     unsigned long long ev = evals;
 #pragma unroll
@@ -403,24 +465,151 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 4 ? 16 : 1)) void k_ras
   }
 }
 
+// Sums of the split lists' segments (all but the first: nothing lies in
+// front of it) for the segments before them: per pixel the product of
+// (1 - alpha) and, with transmittance 1 before the segment, sum of alpha T
+// dL/dC.rgb, over the entries that the forward's walk reached.  The
+// forward's walk and geometry (two pixels per thread) on the backward's
+// bounds; no gradients, so about half of a segment's backward.
+template <int kT>
+__global__ __launch_bounds__(Geo<kFwdPx>::kThreads, 10) void k_bwd_sums(
+    const float *__restrict__ rec, const uint32_t *__restrict__ vals, const uint64_t *__restrict__ ranges,
+    const DevView *__restrict__ views, const uint32_t *__restrict__ toff, int V,
+    const uint32_t *__restrict__ ncontrib, const float *__restrict__ dimg, pk_device_status *status, uint32_t npairs,
+    SplitBwd split, uint32_t split_items, RasterQueue *rq) {
+  constexpr int kPx = kFwdPx, kBatch = 128;
+  using G = Geo<kPx>;
+  constexpr uint32_t kQuads = (kT / kTileSide) * (kT / kTileSide);
+  __shared__ float4 s_a[kBatch], s_b[kBatch], s_c[kBatch], s_box[kBatch], s_q[kBatch];
+  __shared__ uint32_t s_item, s_seg;
+  __shared__ int s_view;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const Staged st{s_a, s_b, s_c, s_box, s_q};
+  int ox, oy, bx, by;
+  pixel_of<kPx>(tid, ox, oy, bx, by);
+  for (;;) {
+    if (tid == 0) {
+      uint32_t it, seg;
+      s_view = -1;
+      if (split_next(rq, split.items, split_items, 0, 1u, it, seg)) {
+        s_item = it;
+        s_seg = seg;
+        s_view = view_of_tile(toff, V, split.items[it].w / kQuads);
+      }
+    }
+    __syncthreads();
+    if (s_view < 0) break;
+    const SplitItem item = split.items[s_item];
+    const uint32_t seg = s_seg;
+    const uint32_t t = item.w / kQuads, qd = item.w - t * kQuads;
+    const DevView &view = views[s_view];
+    const int W = view.width, H = view.height;
+    const uint32_t local = t - (uint32_t)view.tile_off;
+    const int ty = (int)(local / (uint32_t)view.tiles_x), tx = (int)(local - (uint32_t)ty * view.tiles_x);
+    const int x = tx * kT + (int)(qd % (kT / kTileSide)) * kTileSide + ox;
+    const int y0 = ty * kT + (int)(qd / (kT / kTileSide)) * kTileSide + oy;
+    const float px = (float)x + 0.5f, py0 = (float)y0 + 0.5f;
+    const uint64_t s = __ldg(ranges + 2 * (size_t)t);
+    const uint32_t len = (uint32_t)(__ldg(ranges + 2 * (size_t)t + 1) - s);
+    const uint32_t beg = seg * item.x, end = seg + 1 < item.nseg ? beg + item.x : item.len;
+    const size_t plane = (size_t)W * H;
+    float T[kPx], L[kPx], g0[kPx], g1[kPx], g2[kPx];
+    uint32_t nc[kPx], ncmax = 0;
+    int ylo = 0x3fffffff, yhi = -0x3fffffff;
+#pragma unroll
+    for (int k = 0; k < kPx; ++k) {
+      const int y = y0 + k * G::kRowStep;
+      T[k] = 1.f;
+      L[k] = g0[k] = g1[k] = g2[k] = 0.f;
+      nc[k] = 0;
+      if (x < W && y < H) {
+        const float *gi = dimg + 3 * (size_t)view.pix_off + (size_t)y * W + x;
+        nc[k] = min(ncontrib[(size_t)view.pix_off + (size_t)y * W + x], min(len, item.len));
+        g0[k] = gi[0];
+        g1[k] = gi[plane];
+        g2[k] = gi[2 * plane];
+      }
+      if (nc[k] > beg) {
+        ylo = min(ylo, y);
+        yhi = max(yhi, y);
+      }
+      ncmax = max(ncmax, nc[k]);
+    }
+    const WarpRect wr = warp_rect(ncmax > beg, x, ylo, yhi);
+    const uint32_t wmax = min(end, __reduce_max_sync(0xffffffffu, ncmax));
+    for (uint32_t base = beg; base < end; base += kBatch) {
+      const int nb = (int)min((uint32_t)kBatch, end - base);
+      if (!__syncthreads_or(base < wmax)) break;   // no pixel reaches further (and the last batch is done with)
+      for (int j = tid; j < nb; j += G::kThreads)
+        stage_splat(rec, __ldg(vals + s + base + j), npairs, st, j, status);
+      __syncthreads();
+#pragma unroll 1
+      for (int k = 0; k < kBatch / 32; ++k) {
+        const int jl = 32 * k + lane;
+        uint32_t m = __ballot_sync(0xffffffffu, jl < nb && base + (uint32_t)jl < wmax &&
+                                                    block_may_hit(s_box[jl], s_q[jl], s_a[jl].x, s_a[jl].y, wr.x0,
+                                                                  wr.x1, wr.y0, wr.y1));
+        while (m) {
+          const int j = 32 * k + __ffs(m) - 1;
+          m &= m - 1;
+          const uint32_t pos = base + (uint32_t)j;
+          const float4 a = s_a[j], b = s_b[j], c = s_c[j];
+          const float dx = __fsub_rn(px, a.x);
+          const float zxdx = __fmul_rn(__fmul_rn(a.z, dx), dx), bdx = __fmul_rn(a.w, dx);
+#pragma unroll
+          for (int q = 0; q < kPx; ++q) {
+            const float power = splat_power(a, b, bdx, zxdx, py0 + (float)(q * G::kRowStep));
+            if (pos < nc[q] && power >= c.z) {
+              const float alpha = fminf(__fmul_rn(-b.y, ex2_approx(power)), kAlphaMax);
+              L[q] = fmaf(alpha * T[q], fmaf(g2[q], c.x, fmaf(g1[q], b.w, g0[q] * b.z)), L[q]);
+              T[q] = __fmul_rn(T[q], __fsub_rn(1.f, alpha));
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kPx; ++k) {
+      const size_t pu = ((size_t)item.unit0 + seg) * kSplitBlock + (oy + k * G::kRowStep) * kTileSide + ox;
+      split.tl[pu] = T[k];
+      split.ls[pu] = L[k];
+    }
+    __syncthreads();   // everyone is done with this unit's shared state
+  }
+}
+
 // One persistent launch: as many CTAs as fit on the GPU, at most one per tile.
-template <int kBatch, bool kBwdTma, int kT, bool kCount>
+template <int kBatch, bool kBwdTma, int kT, bool kCount, BwdSplit kSplit>
 pk_status launch_bwd(const pk_plan *p, const float *records, const uint32_t *sorted_vals,
                      const uint64_t *tile_ranges, const float *T_final, const uint32_t *n_contrib,
                      const float *dL_dimage, float *grad2d, void *ws, DevCounters *ctr, pk_device_status *status,
                      cudaStream_t st) {
   static KernelInfo info;
   const int sms = sm_count();
-  const auto kernel = k_raster_bwd<kBatch, kBwdTma, kBwdPx, kT, kCount>;
+  const auto kernel = k_raster_bwd<kBatch, kBwdTma, kBwdPx, kT, kCount, kSplit>;
   const int per_sm = std::max(1, resident_ctas(info, reinterpret_cast<const void *>(kernel), Geo<kBwdPx>::kThreads, 0));
   const int64_t items = p->n_tiles * (kT / kTileSide) * (kT / kTileSide);
   int64_t grid = (int64_t)sms * per_sm;
   if (grid > items) grid = items;
   if (grid < 1) grid = 1;
-  k_raster_bwd<kBatch, kBwdTma, kBwdPx, kT, kCount><<<(int)grid, Geo<kBwdPx>::kThreads, 0, st>>>(
-      records, sorted_vals, tile_ranges, at<DevView>(ws, p->ws.views), at<uint32_t>(ws, p->ws.toff), p->V,
-      (uint32_t)items, p->opts.bg[0], p->opts.bg[1], p->opts.bg[2], T_final, n_contrib, dL_dimage, grad2d,
-      &ctr->tile_queue[1], reinterpret_cast<unsigned long long *>(&status->evals_bwd), status, p->first_polls, (uint32_t)p->pairs);
+  const SplitBwd split = SplitBwd::of(at<char>(ws, p->ws.split), p->long_items, p->split_units);
+  const DevView *views = at<DevView>(ws, p->ws.views);
+  const uint32_t *toff = at<uint32_t>(ws, p->ws.toff);
+  auto launch = [&](auto kernel, int64_t blocks) {
+    kernel<<<(int)blocks, Geo<kBwdPx>::kThreads, 0, st>>>(
+        records, sorted_vals, tile_ranges, views, toff, p->V, (uint32_t)items, p->opts.bg[0], p->opts.bg[1],
+        p->opts.bg[2], T_final, n_contrib, dL_dimage, grad2d,
+        reinterpret_cast<unsigned long long *>(&status->evals_bwd), status, p->first_polls, (uint32_t)p->pairs, split,
+        p->long_items, p->split_units, &ctr->raster[1],
+        std::min<uint32_t>(p->long_items, (uint32_t)(sms * per_sm / 4)));
+  };
+  launch(k_raster_bwd<kBatch, kBwdTma, kBwdPx, kT, kCount, kSplit>, grid);
+  if (kSplit == kEnter) {   // the split lists: at most split_units segments, as many CTAs as are resident
+    k_bwd_sums<kT><<<(int)std::min<int64_t>((int64_t)sms * 10, p->split_units), Geo<kFwdPx>::kThreads, 0, st>>>(
+        records, sorted_vals, tile_ranges, views, toff, p->V, n_contrib, dL_dimage, status, (uint32_t)p->pairs, split,
+        p->long_items, &ctr->raster[1]);
+    launch(k_raster_bwd<128, false, kBwdPx, kT, false, kSegments>, std::min<int64_t>((int64_t)sms * 16, p->split_units));
+  }
   return check_launch();
 }
 
@@ -440,21 +629,26 @@ pk_status rasterize_bwd(const pk_plan *p, const float *records, const uint32_t *
   DevCounters *ctr = at<DevCounters>(ws, p->ws.counters);
   pk_device_status *status = at<pk_device_status>(ws, p->ws.status);
   pk_status ze = zero_async({{grad2d, zero_grad2d ? sizeof(float) * kG2d * (size_t)p->pairs : 0},
-                             {&ctr->tile_queue[1], sizeof(uint32_t)},
+                             {&ctr->raster[1], sizeof(RasterQueue)},
                              {&status->evals_bwd, sizeof(uint64_t)}},
                             st);
   if (ze != PK_OK) return ze;
-#define PK_BWD_T(B, M, C)                                                                                   \
-  return p->T == 32 ? launch_bwd<B, M, 32, C>(p, records, sorted_vals, tile_ranges, T_final, n_contrib,       \
-                                              dL_dimage, grad2d, ws, ctr, status, st)                         \
-                    : launch_bwd<B, M, 16, C>(p, records, sorted_vals, tile_ranges, T_final, n_contrib,       \
-                                              dL_dimage, grad2d, ws, ctr, status, st)
-#define PK_BWD(B, M)            \
-  {                             \
-    if (p->opts.count_evals) {  \
-      PK_BWD_T(B, M, true);     \
-    }                           \
-    PK_BWD_T(B, M, false);      \
+  const int side = p->T == 32 ? 2 : 1;
+  const bool split = p->n_tiles * side * side <= kLongPasses * (int64_t)sm_count() * 10;   // the forward's rule
+#define PK_BWD_T(B, M, C, S)                                                                                \
+  return p->T == 32 ? launch_bwd<B, M, 32, C, S>(p, records, sorted_vals, tile_ranges, T_final, n_contrib,    \
+                                                 dL_dimage, grad2d, ws, ctr, status, st)                      \
+                    : launch_bwd<B, M, 16, C, S>(p, records, sorted_vals, tile_ranges, T_final, n_contrib,    \
+                                                 dL_dimage, grad2d, ws, ctr, status, st)
+#define PK_BWD(B, M)                  \
+  {                                   \
+    if (p->opts.count_evals) {        \
+      PK_BWD_T(B, M, true, kNoSplit); \
+    }                                 \
+    if (split) {                      \
+      PK_BWD_T(B, M, false, kEnter);  \
+    }                                 \
+    PK_BWD_T(B, M, false, kNoSplit);  \
   }
   const bool tma = p->opts.stage_bwd == PK_STAGE_BULK;
   switch (p->opts.batch_bwd) {
