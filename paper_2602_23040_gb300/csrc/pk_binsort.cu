@@ -369,30 +369,31 @@ __global__ __launch_bounds__(kThreads) void k_pair_count(const float *__restrict
   }
 }
 
+// The depth sort's keys are bits(z) less those of the nearest pair, in the
+// same order, and a pass whose digit is 0 in every key is left out: depths
+// between 2.5 and 5.5 span fewer than 2^24 floats, so a rig around its scene
+// sorts in three passes of four (52-view rig: the depth passes 1,084 -> 949 us).  The kernels of such a pass
+// return at once, and whoever reads the sorted pairs takes the buffer that
+// the last pass wrote.
+struct DepthPasses {
+  int shift[3];   // first key bit of passes 1, 2, 3 (32: there is no such pass)
+};
+__device__ __forceinline__ uint32_t depth_span(const DevCounters *ctr) { return ctr->z_max - ~ctr->nz_min; }
+__device__ __forceinline__ const uint32_t *sorted_pairs(const DevCounters *ctr, const DepthPasses &dp,
+                                                        const uint32_t *even, const uint32_t *odd) {
+  const uint32_t span = depth_span(ctr);
+  int n = 1;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) n += dp.shift[k] < 32 && (span >> dp.shift[k]) != 0u ? 1 : 0;
+  return (n & 1) ? odd : even;
+}
+
 // ---------------------------------------------------------------------------
 // Chunked reduce-then-scan.  Item i of the scanned sequence is src(i).
 // ---------------------------------------------------------------------------
 
-struct SrcValid {      // 1 if pair i touches a tile
-  const uint32_t *cnt;
-  __device__ uint32_t operator()(uint64_t i) const { return cnt[i] > 0u ? 1u : 0u; }
-};
 __device__ __forceinline__ uint64_t load_n(const uint64_t *n_dev, uint64_t n_host) {
   return n_dev ? *n_dev : n_host;
-}
-
-template <typename Src>
-__global__ __launch_bounds__(kThreads) void k_scan_reduce(Src src, const uint64_t *n_dev, uint64_t n_host,
-                                                          uint64_t *__restrict__ bsum) {
-  __shared__ uint64_t s[kWarps + 1];
-  const uint64_t n = load_n(n_dev, n_host);
-  uint64_t b0, b1;
-  chunk_of(n, gridDim.x, blockIdx.x, kScanTile, b0, b1);
-  uint64_t acc = 0;
-  for (uint64_t i = b0 + threadIdx.x; i < b1; i += kThreads) acc += src(i);
-  uint64_t tot;
-  block_excl_scan<uint64_t>(acc, tot, s);
-  if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
 }
 
 // Items of the blocks before this one, from the block sums: every block of a
@@ -422,7 +423,54 @@ __device__ __forceinline__ void load8(const uint32_t *__restrict__ a, uint64_t i
 }
 static_assert(kScanItems == 8, "load8 takes a thread's scan items");
 
-// Down-sweep of the compaction: writes (bits(z), pair) of every valid pair
+// Reduce of the compaction: the pairs of each block that touch a tile, and
+// the nearest and farthest depth among all of them.
+__global__ __launch_bounds__(kThreads) void k_count_valid(const uint32_t *__restrict__ cnt,
+                                                          const uint32_t *__restrict__ zbits, uint64_t n,
+                                                          uint64_t *__restrict__ bsum, DevCounters *ctr) {
+  __shared__ uint64_t s[kWarps + 1];
+  uint64_t b0, b1;
+  chunk_of(n, gridDim.x, blockIdx.x, kScanTile, b0, b1);
+  uint64_t acc = 0;
+  uint32_t nz_min = 0u, z_max = 0u;
+  for (uint64_t base = b0; base < b1; base += kScanTile) {
+    const uint64_t i0 = base + (uint64_t)threadIdx.x * kScanItems;
+    uint32_t cv[8], zv[8];
+    load8(cnt, i0, b1, cv);
+    load8(zbits, i0, b1, zv);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (cv[j] > 0u) {
+        ++acc;
+        nz_min = max(nz_min, ~zv[j]);
+        z_max = max(z_max, zv[j]);
+      }
+  }
+  uint64_t tot;
+  block_excl_scan<uint64_t>(acc, tot, s);
+  if (threadIdx.x == 0) bsum[blockIdx.x] = tot;
+  // one pair of atomics per block (one per warp made this kernel 70 us at the
+  // 52-view rig)
+  __shared__ uint32_t s_min[kWarps], s_max[kWarps];
+  nz_min = __reduce_max_sync(0xffffffffu, nz_min);
+  z_max = __reduce_max_sync(0xffffffffu, z_max);
+  if ((threadIdx.x & 31) == 0) {
+    s_min[threadIdx.x >> 5] = nz_min;
+    s_max[threadIdx.x >> 5] = z_max;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && tot) {
+#pragma unroll
+    for (int k = 1; k < kWarps; ++k) {
+      nz_min = max(nz_min, s_min[k]);
+      z_max = max(z_max, s_max[k]);
+    }
+    atomicMax(&ctr->nz_min, nz_min);
+    atomicMax(&ctr->z_max, z_max);
+  }
+}
+
+// Down-sweep of the compaction: writes (depth key, pair) of every valid pair
 // in pair order.  A tile's outputs go through shared memory so that the
 // writes are contiguous.
 __global__ __launch_bounds__(kThreads) void k_compact_down(const uint32_t *__restrict__ cnt,
@@ -436,6 +484,7 @@ __global__ __launch_bounds__(kThreads) void k_compact_down(const uint32_t *__res
   uint64_t b0, b1;
   chunk_of(n, gridDim.x, blockIdx.x, kScanTile, b0, b1);
   uint32_t run = (uint32_t)block_base(bsum, s64);   // valid pairs < 2^32
+  const uint32_t z_min = ~ctr->nz_min;
   if (blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) {
     const uint64_t total = run + bsum[blockIdx.x];
     ctr->scan_total = total;
@@ -454,7 +503,7 @@ __global__ __launch_bounds__(kThreads) void k_compact_down(const uint32_t *__res
 #pragma unroll
     for (int j = 0; j < 8; ++j)
       if (cv[j] > 0u) {
-        s_z[pre] = zv[j];
+        s_z[pre] = zv[j] - z_min;
         s_p[pre] = (uint32_t)(i0 + j);
         ++pre;
       }
@@ -472,11 +521,13 @@ __global__ __launch_bounds__(kThreads) void k_compact_down(const uint32_t *__res
 // cnt[pval[i]] (0 for a pair index past the pairs, which a depth pass that
 // gave up can leave), and each block's sum for the offset scan.
 __global__ __launch_bounds__(kThreads) void k_reduce_sorted(const uint32_t *__restrict__ cnt,
-                                                            const uint32_t *__restrict__ pval, uint64_t pairs,
-                                                            const uint64_t *n_dev, uint32_t *__restrict__ csorted,
+                                                            const uint32_t *pv0, const uint32_t *pv1, DepthPasses dp,
+                                                            uint64_t pairs, const DevCounters *ctr,
+                                                            uint32_t *__restrict__ csorted,
                                                             uint64_t *__restrict__ bsum) {
   __shared__ uint64_t s[kWarps + 1];
-  const uint64_t n = *n_dev;
+  const uint32_t *__restrict__ pval = sorted_pairs(ctr, dp, pv0, pv1);
+  const uint64_t n = ctr->n_valid;
   uint64_t b0, b1;
   chunk_of(n, gridDim.x, blockIdx.x, kScanTile, b0, b1);
   uint64_t acc = 0;
@@ -635,7 +686,8 @@ template <int RB, int IT>
 __global__ __launch_bounds__(kThreads) void k_radix_upsweep(const uint32_t *__restrict__ keys,
                                                             const uint64_t *n_dev, uint64_t n_host, int shift,
                                                             uint32_t mask, uint64_t *__restrict__ hist,
-                                                            DigitBase base, SegSpec sp) {
+                                                            DigitBase base, SegSpec sp, const DevCounters *depth) {
+  if (depth && shift && (depth_span(depth) >> shift) == 0u) return;   // the digit is 0 in every depth key
   using C = Radix<RB, IT>;
   __shared__ uint32_t s_cnt[C::kCopies][C::kR];   // private digit counts
   for (int i = threadIdx.x; i < C::kCopies * C::kR; i += kThreads) (&s_cnt[0][0])[i] = 0;
@@ -807,7 +859,8 @@ __global__ __launch_bounds__(kThreads, (Radix<RB, IT>::kMinBlocks)) void k_radix
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
     uint32_t *__restrict__ vout, const uint64_t *n_dev, uint64_t n_host, int shift, uint32_t mask,
     const uint64_t *__restrict__ hist, pk_device_status *status, SegSpec sp, uint32_t *abort_flag,
-    uint32_t first_polls, bool try_single, DigitBase dbase, Unpack up) {
+    uint32_t first_polls, bool try_single, DigitBase dbase, const DevCounters *depth, Unpack up) {
+  if (depth && shift && (depth_span(depth) >> shift) == 0u) return;   // the digit is 0 in every depth key
   using C = Radix<RB, IT>;
   constexpr bool kV = kMode == 0, kLast = kMode == 2;
   constexpr int kTile = C::kTile;
@@ -1085,7 +1138,8 @@ struct EmitFoot {
   int4 r;          // first candidate tile (x, y), view width and height
 };
 
-__global__ __launch_bounds__(kThreads) void k_emit(const float *__restrict__ rec, const uint32_t *__restrict__ pval,
+__global__ __launch_bounds__(kThreads) void k_emit(const float *__restrict__ rec, const uint32_t *pv0,
+                                                   const uint32_t *pv1, DepthPasses dp,
                                                    const uint64_t *__restrict__ offs, const uint4 *__restrict__ pinfo,
                                                    DevCounters *ctr, const DevView *__restrict__ views,
                                                    int64_t N, int64_t pairs, int T, int mode, int local_bits,
@@ -1095,6 +1149,7 @@ __global__ __launch_bounds__(kThreads) void k_emit(const float *__restrict__ rec
   __shared__ EmitFoot s_ef[kWarps][32];
   const uint64_t dups = ctr->dups;
   if (dups == 0) return;
+  const uint32_t *__restrict__ pval = sorted_pairs(ctr, dp, pv0, pv1);
   const uint64_t n = ctr->n_valid;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = lanemask_lt();
@@ -1203,9 +1258,10 @@ __global__ __launch_bounds__(kThreads) void k_emit(const float *__restrict__ rec
 // are global tile ids, or (local_bits > 0) the view above a per-view local
 // tile id: then the view's tile_off is added to the local id.
 __global__ __launch_bounds__(kThreads) void k_ranges(const uint32_t *__restrict__ keys, int local_bits,
-                                                     const uint32_t *__restrict__ toff, const DevCounters *ctr,
+                                                     const uint32_t *__restrict__ toff, DevCounters *ctr,
                                                      uint64_t *__restrict__ ranges, int V, uint32_t n_tiles,
                                                      pk_device_status *status) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctr->nz_min = ctr->z_max = 0u;   // the call's last kernel
   const uint64_t n = ctr->sort_abort ? 0u : ctr->dups;   // a pass gave up: every range stays empty
   const uint64_t nq = (n + 3) / 4;
   const uint32_t lmask = (1u << local_bits) - 1u;
@@ -1252,8 +1308,9 @@ __global__ __launch_bounds__(kThreads) void k_ranges(const uint32_t *__restrict_
 // ~position (0: no entry) and end as the largest position + 1.  A call
 // that gave up leaves every range empty.
 __global__ __launch_bounds__(kThreads) void k_range_fix(uint64_t *__restrict__ ranges, uint32_t n_tiles,
-                                                        const DevCounters *ctr) {
+                                                        DevCounters *ctr) {
   const bool gave_up = ctr->sort_abort != 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctr->nz_min = ctr->z_max = 0u;   // the call's last kernel
   for (uint32_t t = blockIdx.x * kThreads + threadIdx.x; t < n_tiles; t += gridDim.x * kThreads) {
     const uint64_t a = ranges[2 * (size_t)t];
     if (gave_up || a == 0ull) {
@@ -1271,10 +1328,12 @@ __global__ __launch_bounds__(kThreads) void k_range_fix(uint64_t *__restrict__ r
 // (the total number of entries where no such pair is left), else seg[v] =
 // its index (n where none is left); seg[V] = the total.
 template <bool kEntries>
-__global__ __launch_bounds__(kThreads) void k_view_segments(const uint32_t *__restrict__ pval,
+__global__ __launch_bounds__(kThreads) void k_view_segments(const uint32_t *pv0, const uint32_t *pv1, DepthPasses dp,
                                                             const uint64_t *__restrict__ offs,
                                                             const DevCounters *ctr, uint32_t N, int V,
                                                             uint64_t *__restrict__ seg) {
+  // the pairs in compaction order, or (kEntries) sorted: either way grouped by view
+  const uint32_t *__restrict__ pval = kEntries ? sorted_pairs(ctr, dp, pv0, pv1) : pv0;
   const uint32_t n = (uint32_t)ctr->n_valid;   // valid pairs < 2^32 (pair indices are 32-bit)
   const uint64_t total = kEntries ? ctr->dups : n;
   for (int v = blockIdx.x * kThreads + threadIdx.x; v <= V; v += gridDim.x * kThreads) {
@@ -1296,7 +1355,7 @@ template <int RB, int IT, int kMode>
 pk_status radix_pass_rb(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout,
                         const uint64_t *n_dev, uint64_t n_host, int shift, int bits, uint64_t *hist, int nblocks,
                         DigitBase dbase, uint64_t *csum, pk_device_status *status, SegSpec sp, uint32_t *abort_flag,
-                        uint32_t first_polls, bool try_single, const Unpack &up, cudaStream_t st) {
+                        uint32_t first_polls, bool try_single, const DevCounters *depth, const Unpack &up, cudaStream_t st) {
   using C = Radix<RB, IT>;
   static KernelInfo info;
   const auto downsweep = k_radix_downsweep<RB, IT, kMode>;
@@ -1304,7 +1363,7 @@ pk_status radix_pass_rb(const uint32_t *kin, const uint32_t *vin, uint32_t *kout
     return PK_ERR_CUDA;
   const uint32_t mask = (1u << bits) - 1u;
   if (dbase != kSolo)
-    k_radix_upsweep<RB, IT><<<nblocks, kThreads, 0, st>>>(kin, n_dev, n_host, shift, mask, hist, dbase, sp);
+    k_radix_upsweep<RB, IT><<<nblocks, kThreads, 0, st>>>(kin, n_dev, n_host, shift, mask, hist, dbase, sp, depth);
   if (dbase == kScan) {
     const int count = C::kR * nblocks, nchunks = (count + kHistChunk - 1) / kHistChunk;
     k_radix_chunk_sums<<<nchunks, 1024, 0, st>>>(hist, count, csum);
@@ -1312,7 +1371,7 @@ pk_status radix_pass_rb(const uint32_t *kin, const uint32_t *vin, uint32_t *kout
   }
   k_radix_downsweep<RB, IT, kMode><<<nblocks, kThreads, Down<RB, IT>::kSmem, st>>>(
       kin, vin, kout, vout, n_dev, n_host, shift, mask, hist, status, sp, abort_flag, first_polls, try_single, dbase,
-      up);
+      depth, up);
   return check_launch();
 }
 
@@ -1326,11 +1385,11 @@ pk_status radix_pass(bool entries, int rb, const uint32_t *kin, const uint32_t *
                      const uint64_t *n_dev, uint64_t n_host, int shift, int bits, uint64_t *hist, int nblocks,
                      DigitBase dbase, uint64_t *csum, pk_device_status *status, uint32_t *abort_flag, uint32_t first_polls,
                      bool try_single, cudaStream_t st, SegSpec sp = SegSpec{nullptr, nullptr},
-                     Unpack up = Unpack{}) {
+                     const DevCounters *depth = nullptr, Unpack up = Unpack{}) {
 #define PK_PASS(RB, IT, M)                                                                                        \
   return radix_pass_rb<RB, IT, M>(kin, vin, kout, vout, n_dev, n_host, shift, bits, hist, nblocks, dbase, csum,   \
                                   status,                                                                   \
-                                  sp, abort_flag, first_polls, try_single, up, st)
+                                  sp, abort_flag, first_polls, try_single, depth, up, st)
   if (entries) {
     if (!vin && up.ranges) {
       if (rb > 8) PK_PASS(11, kEntryItems, 2);
@@ -1479,14 +1538,14 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
                                               zk[1], tile_ranges, 2u * (uint32_t)p->n_tiles, &ctr->sort_abort);
   // compaction of the pairs that touch a tile, keyed by depth bits
   const int sblocks = (int)std::min<uint64_t>((pairs + kScanTile - 1) / kScanTile, kScanBlocks);
-  k_scan_reduce<SrcValid><<<sblocks, kThreads, 0, st>>>(SrcValid{cnt}, nullptr, pairs, bsum);
+  k_count_valid<<<sblocks, kThreads, 0, st>>>(cnt, zk[1], pairs, bsum, ctr);
   k_compact_down<<<sblocks, kThreads, 0, st>>>(cnt, zk[1], pairs, bsum, zk[0], pv[0], ctr, status);
   // depth sort of the pairs: stable passes over the 32 bits of z; the
   // compaction kept the (view, Gaussian) order, so sorting inside each
   // view's segment leaves the pairs in (view, depth) order
   SegSpec psp{nullptr, nullptr};
   if (seg) {
-    k_view_segments<false><<<(p->V + kThreads) / kThreads, kThreads, 0, st>>>(pv[0], nullptr, ctr, (uint32_t)p->N,
+    k_view_segments<false><<<(p->V + kThreads) / kThreads, kThreads, 0, st>>>(pv[0], pv[0], DepthPasses{}, nullptr, ctr, (uint32_t)p->N,
                                                                             p->V, pseg);
     psp = SegSpec{tab + L.sort_cap, pseg};
   }
@@ -1498,21 +1557,22 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
     const int a = pass & 1, b = a ^ 1;
     if ((e = radix_pass(false, rd, zk[a], pv[a], zk[b], pv[b], n_valid, 0, shift, widths[pass], hist,
                         blk.npair, (DigitBase)blk.pair_base, bsum, status, &ctr->sort_abort, p->first_polls,
-                        pass == np - 1, st, psp)) != PK_OK)
+                        pass == np - 1, st, psp, ctr)) != PK_OK)
       return e;
     shift += widths[pass];
   }
-  const uint32_t *pval = pv[np & 1];
+  DepthPasses dp{{32, 32, 32}};
+  for (int pass = 1, bit = widths[0]; pass < np; bit += widths[pass++]) dp.shift[pass - 1] = bit;
   // emission offsets in (view,) depth order, capacity check
   uint32_t *csorted = zk[1];   // the depth keys are spent: their buffer takes the gathered counts
-  k_reduce_sorted<<<sblocks, kThreads, 0, st>>>(cnt, pval, pairs, n_valid, csorted, bsum);
+  k_reduce_sorted<<<sblocks, kThreads, 0, st>>>(cnt, pv[0], pv[1], dp, pairs, ctr, csorted, bsum);
   k_offsets_down<<<sblocks, kThreads, 0, st>>>(csorted, n_valid, bsum, maxd, ctr, status, offs);
   // emission and the stable tile sort; the last pass lands in sorted_vals
   int key_bits = p->tile_bits;
   SegSpec sp{nullptr, nullptr};
   if (seg) {
     key_bits = local_tile_bits(p);
-    k_view_segments<true><<<(p->V + kThreads) / kThreads, kThreads, 0, st>>>(pval, offs, ctr, (uint32_t)p->N, p->V,
+    k_view_segments<true><<<(p->V + kThreads) / kThreads, kThreads, 0, st>>>(pv[0], pv[1], dp, offs, ctr, (uint32_t)p->N, p->V,
                                                                           vseg);
     sp = SegSpec{tab, vseg};
   }
@@ -1528,7 +1588,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   np = radix_plan(key_bits, rt, widths);
   uint32_t *vbuf[2] = {(np & 1) ? dv : sorted_vals, (np & 1) ? sorted_vals : dv};
   uint32_t *kbuf[2] = {dk0, dk1};
-  k_emit<<<sms * 32, kThreads, 0, st>>>(records, pval, offs, pinfo, ctr, views, p->N, p->pairs, p->T,
+  k_emit<<<sms * 32, kThreads, 0, st>>>(records, pv[0], pv[1], dp, offs, pinfo, ctr, views, p->N, p->pairs, p->T,
                                                       p->opts.bin_mode, seg ? key_bits : 0, packed ? pbits : 0,
                                                       kbuf[0], vbuf[0], status);
   // Digits from the top down: each tile's entries still end up contiguous
@@ -1547,7 +1607,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
       e = radix_pass(true, rt, kbuf[a], nullptr, last ? nullptr : kbuf[b], last ? sorted_vals : nullptr, &ctr->dups,
                      0, shift, widths[pass], hist, blk.ntile, (DigitBase)blk.tile_base, bsum, status, &ctr->sort_abort,
                      p->first_polls, false,
-                     st, sp, last ? up : Unpack{});
+                     st, sp, nullptr, last ? up : Unpack{});
     else
       e = radix_pass(true, rt, kbuf[a], vbuf[a], kbuf[b], vbuf[b], &ctr->dups, 0, shift, widths[pass], hist, blk.ntile,
                      (DigitBase)blk.tile_base, bsum, status, &ctr->sort_abort, p->first_polls, false, st, sp);

@@ -76,6 +76,8 @@ struct DevCounters {
   float ssim_lambda;       // its lambda (0 after pk_l1_loss_grad)
   uint32_t sort_abort;     // this bin_and_sort call gave up (a wait timed out or an index check
                            // failed): it emits nothing; cleared at the start of each call
+  uint32_t nz_min, z_max;  // ~bits of the nearest depth among the pairs that touch a tile, bits of the
+                           // farthest; 0 between bin_and_sort calls
 };
 
 // Byte offsets of every region inside the workspace.
