@@ -40,9 +40,11 @@ __global__ __launch_bounds__(kProjThreads) void k_project(const float *__restric
         finite = finite && isfinite(kv);
       }
     const int vb = __ldg(fview_off + f), ve = __ldg(fview_off + f + 1);
+    int nv = vb < ve ? __ldg(fview_idx + vb) : 0;   // the next view, read a view ahead
     for (int vi = vb; vi < ve; ++vi) {
-      const int v = __ldg(fview_idx + vi);
-      const DevView &view = views[v];
+      const int v = nv;
+      const ViewCam view = load_cam(views + v);
+      if (vi + 1 < ve) nv = __ldg(fview_idx + vi + 1);
       float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0, r2 = r0;
       Proj p;
       bool ok = finite && project(a, view, znear, p);
