@@ -198,6 +198,13 @@ __global__ __launch_bounds__(kMaskThreads) void k_mask_coarse(const uint32_t *__
   if (lane == 0) coarse[view.coarse_off + w] = word;
 }
 
+// d^2 of a pixel in FP32 without fused multiply-adds, in the order stated in
+// packuv.h (b2 = 2 b).
+__device__ __forceinline__ float pixel_q(float a, float c, float b2, float dx, float dy) {
+  return __fadd_rn(__fadd_rn(__fmul_rn(__fmul_rn(a, dx), dx), __fmul_rn(__fmul_rn(c, dy), dy)),
+                   __fmul_rn(__fmul_rn(b2, dy), dx));
+}
+
 // Does the ellipse q <= 9 of a pair cover a moving pixel of its rectangle
 // [x0, x1] x [y0, y1]?  Called by a whole warp with the same pair: lane l
 // takes rows y0 + l, y0 + l + 32, ...; per row a conservative filter keeps
@@ -243,7 +250,6 @@ __device__ bool warp_pair_hits(float mx, float my, float a, float b, float c, in
         xb = min(xb, (int)fminf(floorf(xc + half), (float)(W - 1)));
       }
       if (xa <= xb) {
-        const float cyy = __fmul_rn(__fmul_rn(c, dy), dy), bdy = __fmul_rn(b2, dy);
         const int wa = xa >> 5, wb = xb >> 5;
         for (int wx = wa; wx <= wb && !h; ++wx) {
           if (!((__ldg(crow + (wx >> 5)) >> (wx & 31)) & 1u)) continue;
@@ -254,8 +260,7 @@ __device__ bool warp_pair_hits(float mx, float my, float a, float b, float c, in
             const int x = 32 * wx + __ffs(m) - 1;
             m &= m - 1u;
             const float dx = __fsub_rn(__fadd_rn((float)x, 0.5f), mx);
-            const float q = __fadd_rn(__fadd_rn(__fmul_rn(__fmul_rn(a, dx), dx), cyy), __fmul_rn(bdy, dx));
-            if (q <= kQMax) {
+            if (pixel_q(a, c, b2, dx, dy) <= kQMax) {
               h = true;
               break;
             }
@@ -291,7 +296,7 @@ __device__ __forceinline__ bool block_moves(const uint32_t *__restrict__ vcoarse
 // its own pair: the block mask over the square of radius r around the mean,
 // and where that moves the conservative extent filter (rows within
 // 3 sqrt(a / det) of the mean, columns within 3 sqrt(c / det), widened) and
-// the block mask over that rectangle.  The extents take the one-instruction
+// the block mask over that rectangle, then the pixel at the mean.  The extents take the one-instruction
 // reciprocal and root: their relative error near 2^-22 is far below the
 // widening, so they too only ever skip what cannot pass (607 -> 549 us at
 // the 52-view rig with the square tested first and, in the scan, the mask's
@@ -362,6 +367,23 @@ __global__ __launch_bounds__(kMaskThreads) void k_dynamic_mask(const float *__re
         }
       }
     }
+    auto mark = [&]() {
+      const uint32_t ty = t / (uint32_t)atlas_w, tx = t - ty * (uint32_t)atlas_w;
+      atomicOr(dyn + (size_t)ty * (((uint32_t)atlas_w + 31u) >> 5) + (tx >> 5), 1u << (tx & 31u));
+      live = false;
+    };
+    if (need) {
+      // a Gaussian inside the moving region: the pixel at its mean decides,
+      // by the scan's own test, and spares the scan
+      const int x = min(max((int)rintf(__fsub_rn(mx, 0.5f)), x0), x1), y = min(max((int)rintf(__fsub_rn(my, 0.5f)), y0), y1);
+      if ((__ldg(vmask + (int64_t)y * wpr + (x >> 5)) >> (x & 31)) & 1u) {
+        const float dx = __fsub_rn(__fadd_rn((float)x, 0.5f), mx), dy = __fsub_rn(__fadd_rn((float)y, 0.5f), my);
+        if (pixel_q(a, c, __fmul_rn(2.0f, b), dx, dy) <= kQMax) {
+          mark();
+          need = false;
+        }
+      }
+    }
     uint32_t todo = __ballot_sync(0xffffffffu, need);
     while (todo) {
       const int src = __ffs(todo) - 1;
@@ -371,12 +393,8 @@ __global__ __launch_bounds__(kMaskThreads) void k_dynamic_mask(const float *__re
       const float sc = __shfl_sync(0xffffffffu, c, src);
       const int sx0 = __shfl_sync(0xffffffffu, x0, src), sx1 = __shfl_sync(0xffffffffu, x1, src);
       const int sy0 = __shfl_sync(0xffffffffu, y0, src), sy1 = __shfl_sync(0xffffffffu, y1, src);
-      if (warp_pair_hits(smx, smy, sa, sb, sc, sx0, sx1, sy0, sy1, W, wpr, cpr, vmask, vcoarse, lane) &&
-          lane == src) {
-        const uint32_t ty = t / (uint32_t)atlas_w, tx = t - ty * (uint32_t)atlas_w;
-        atomicOr(dyn + (size_t)ty * (((uint32_t)atlas_w + 31u) >> 5) + (tx >> 5), 1u << (tx & 31u));
-        live = false;
-      }
+      if (warp_pair_hits(smx, smy, sa, sb, sc, sx0, sx1, sy0, sy1, W, wpr, cpr, vmask, vcoarse, lane) && lane == src)
+        mark();
     }
   }
 }
