@@ -159,9 +159,9 @@ __device__ __forceinline__ void activate(const Get &attr, Act &a) {
 }
 
 // What projection and colour need of a view, read in five 16-byte loads (a
-// warp's lanes share them) instead of a load per number: in the kernels that
-// walk the views, waiting for those was the top stall (projection of the
-// 52-view rig 525 -> 474 us).
+// warp's lanes share them) instead of a load per number: in the projection,
+// waiting for those was the top stall (52-view rig 525 -> 474 us; the
+// scatter, which waits for its gradients, is no faster for it).
 struct ViewCam {
   float R[9], t[3];
   float fx, fy, cx, cy;
@@ -187,7 +187,8 @@ struct Proj {
   float radius;
 };
 
-__device__ __forceinline__ bool project(const Act &a, const ViewCam &v, float znear, Proj &p) {
+template <typename View>   // DevView or ViewCam
+__device__ __forceinline__ bool project(const Act &a, const View &v, float znear, Proj &p) {
   const float *W = v.R;
   p.X[0] = W[0] * a.mu[0] + W[1] * a.mu[1] + W[2] * a.mu[2] + v.t[0];
   p.X[1] = W[3] * a.mu[0] + W[4] * a.mu[1] + W[5] * a.mu[2] + v.t[1];
@@ -230,7 +231,8 @@ __device__ __forceinline__ bool project(const Act &a, const ViewCam &v, float zn
 }
 
 // Unit viewing direction and its length.
-__device__ __forceinline__ void view_dir(const Act &a, const ViewCam &v, float *d, float &len) {
+template <typename View>
+__device__ __forceinline__ void view_dir(const Act &a, const View &v, float *d, float &len) {
   float u0 = a.mu[0] - v.campos[0], u1 = a.mu[1] - v.campos[1], u2 = a.mu[2] - v.campos[2];
   len = sqrtf(u0 * u0 + u1 * u1 + u2 * u2);
   const float il = 1.f / len;

@@ -81,7 +81,7 @@ __global__ __launch_bounds__(kScatterThreads, 4) void k_scatter(const float *__r
       if (g0.x == 0.f && g0.y == 0.f && g0.z == 0.f && g0.w == 0.f && g1.x == 0.f && g1.y == 0.f &&
           g1.z == 0.f && g1.w == 0.f && g2.x == 0.f)
         continue;
-      const ViewCam view = load_cam(views + v);
+      const DevView &view = views[v];
       Proj p;
       if (!project(a, view, znear, p)) continue;
       // colour: rgb = max(0, sum_j k_j Y_j(dir) + 0.5)
