@@ -4,7 +4,7 @@
 // Contract: entries ordered by (global tile id, bits(z), pair index).
 // Instead of sorting (tile << 32 | bits(z)) keys over all entries, which
 // costs about 7 radix passes over every (pair, tile) entry, the pairs are
-// first sorted by depth alone (4 passes over pairs, ~15x fewer than
+// first sorted by depth alone (3 or 4 passes over pairs, far fewer than
 // entries), entries are emitted in that depth order, and a stable sort on
 // the tile id alone (ceil(log2 tiles) bits, 2-3 passes) finishes the job:
 // inside one tile every entry comes from the same view, so the stable

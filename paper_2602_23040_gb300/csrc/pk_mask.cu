@@ -296,12 +296,12 @@ __device__ __forceinline__ bool block_moves(const uint32_t *__restrict__ vcoarse
 // its own pair: the block mask over the square of radius r around the mean,
 // and where that moves the conservative extent filter (rows within
 // 3 sqrt(a / det) of the mean, columns within 3 sqrt(c / det), widened) and
-// the block mask over that rectangle, then the pixel at the mean.  The extents take the one-instruction
-// reciprocal and root: their relative error near 2^-22 is far below the
-// widening, so they too only ever skip what cannot pass (607 -> 549 us at
-// the 52-view rig with the square tested first and, in the scan, the mask's
-// words before the ellipse's rows).  The
-// pairs whose rectangle reaches a moving block are then scanned one after
+// the block mask over that rectangle, then the pixel at the mean.  The
+// extents take the one-instruction reciprocal and root: their relative
+// error near 2^-22 is far below the widening, so they too only ever skip
+// what cannot pass.  At the 52-view rig 607 -> 549 us with the square tested
+// first and, in the scan, the mask's words before the ellipse's rows, and
+// 534 us with the pixel at the mean.  The pairs whose rectangle reaches a moving block are then scanned one after
 // the other by the whole warp (warp_pair_hits), so that a long scan near
 // the motion does not run on one lane while the others wait.  A Gaussian
 // is marked at its first hit and takes no further views.
