@@ -8,6 +8,7 @@
 #include <cuda_fp16.h>
 
 #include "pk_common.cuh"
+#include "pk_lpo.cuh"
 
 using namespace pk;
 
@@ -204,13 +205,6 @@ __device__ __forceinline__ float lpo_proxy(uint32_t q, float lo, float delta) {
   return __fadd_rn(lo, __fmul_rn((float)q, delta));
 }
 
-__device__ __forceinline__ uint32_t lpo_code(float x, float lo, float delta, float L) {
-  const float u = floorf(__fadd_rn(__fdiv_rn(__fsub_rn(x, lo), delta), 0.5f));
-  if (!(u >= 0.0f)) return 0u;
-  if (u >= L) return (uint32_t)L;
-  return (uint32_t)u;
-}
-
 // One thread per 4 consecutive texels of a row and group of kChannels
 // channels (blockIdx.y = (frame, group)), whose loads are issued together.
 // kVec: the codes of four texels are one 4-byte load per plane.  At the
@@ -224,11 +218,12 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
                                                     const uint32_t *__restrict__ woff, int W, int H, int F, int D,
                                                     int64_t N, float *__restrict__ soa,
                                                     uint32_t *__restrict__ texel, uint8_t *__restrict__ dynflag) {
-  __shared__ float s_lo[PK_MAX_CHANNELS], s_delta[PK_MAX_CHANNELS];
+  __shared__ float s_lo[PK_MAX_CHANNELS], s_delta[PK_MAX_CHANNELS], s_rd[kCodes ? 1 : PK_MAX_CHANNELS];
   for (int c = threadIdx.x; c < D; c += blockDim.x) {
     const float L = c < 3 ? 65535.0f : 255.0f;
     s_lo[c] = lohi[2 * c];
     s_delta[c] = __fdiv_rn(__fsub_rn(lohi[2 * c + 1], lohi[2 * c]), L);
+    if (!kCodes) s_rd[c] = lpo_rstep(s_delta[c]);
   }
   __syncthreads();
   const uint32_t Wq = (uint32_t)(W + 3) / 4, nq = Wq * (uint32_t)H;
@@ -273,6 +268,7 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
           }
         }
       } else {
+        const uint32_t lanes = (live[0] ? 1u : 0u) | (live[1] ? 2u : 0u) | (live[2] ? 4u : 0u) | (live[3] ? 8u : 0u);
 #pragma unroll 4
         for (int c = c0; c < min(c0 + kChannels, D); ++c) {
           const float lo = s_lo[c], delta = s_delta[c];
@@ -286,10 +282,11 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
             for (int i = 0; i < 4; ++i)
               if (live[i]) x[i] = __ldg(sc + i);
           }
+          uint32_t q[4];
+          lpo_codes4(x, lanes, lo, delta, s_rd[c], c < 3 ? 65535.0f : 255.0f, q);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            if (live[i])
-              dst[(int64_t)c * G + gidx[i]] = lpo_proxy(lpo_code(x[i], lo, delta, c < 3 ? 65535.0f : 255.0f), lo, delta);
+            if (live[i]) dst[(int64_t)c * G + gidx[i]] = lpo_proxy(q[i], lo, delta);
         }
       }
     }

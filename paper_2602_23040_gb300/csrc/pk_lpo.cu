@@ -10,8 +10,10 @@
 // additions (a 64-bit division per group cost more issue slots than the
 // rest of the loop), and the grid is several waves of short blocks, so that
 // no block is left over for a wave of its own.  1024^2 atlas, 59
-// channels: min / max 105 -> 55 us, encode 144 -> 97 us.
+// channels: min / max 105 -> 55 us, encode 144 -> 97 us, and 82 us with the
+// four codes of a group formed without branches (pk_lpo.cuh).
 #include "pk_common.cuh"
+#include "pk_lpo.cuh"
 
 using namespace pk;
 
@@ -157,25 +159,6 @@ __global__ void k_minmax_final(uint32_t *keys, int D) {
   out[2 * c + 1] = none ? 0.0f : unordered(hi);
 }
 
-__device__ __forceinline__ uint32_t lpo_code(float x, float lo, float delta, float L) {
-  const float u = floorf(__fadd_rn(__fdiv_rn(__fsub_rn(x, lo), delta), 0.5f));
-  if (!(u >= 0.0f)) return 0u;
-  if (u >= L) return (uint32_t)L;
-  return (uint32_t)u;
-}
-
-// lpo_code by a multiplication with rd = 1 / delta where that is certain to
-// give the same code: x - lo is the same value, the product lies within
-// 2^-23 relative of the quotient and the sum within 2 x 2^-24, so a sum
-// further than 1e-6 (1 + u) from an integer has the quotient form's floor.
-// The division otherwise (position channels 2 lanes in 100, the others 3 in
-// 10,000), and for a step whose reciprocal loses precision (rd NaN).
-__device__ __forceinline__ uint32_t lpo_code_mul(float x, float lo, float delta, float rd, float L) {
-  const float u = __fadd_rn(__fmul_rn(__fsub_rn(x, lo), rd), 0.5f), fl = floorf(u), m = fmaf(1e-6f, u, 1e-6f);
-  if (u > 0.f && u - fl > m && u - fl < 1.f - m) return (uint32_t)fminf(fl, L);
-  return lpo_code(x, lo, delta, L);
-}
-
 __device__ __forceinline__ void encode_plane(const float *__restrict__ atlas, const uint32_t *__restrict__ occ,
                                              const float *__restrict__ lohi, int W, int H, int D, int64_t fc,
                                              uint8_t *__restrict__ codes) {
@@ -184,7 +167,7 @@ __device__ __forceinline__ void encode_plane(const float *__restrict__ atlas, co
   const float L = c < 3 ? 65535.0f : 255.0f;
   const float lo = __ldg(lohi + 2 * c);
   const float delta = __fdiv_rn(__fsub_rn(__ldg(lohi + 2 * c + 1), lo), L);
-  const float rd = delta > 1e-30f && delta < 1e30f ? __frcp_rn(delta) : __int_as_float(0x7fffffff);
+  const float rd = lpo_rstep(delta);
   const float *src = atlas + fc * plane;
   uint8_t *p0 = codes + ((int64_t)f * (D + 3) + (c < 3 ? 2 * c : c + 3)) * plane;
   uint8_t *p1 = c < 3 ? p0 + plane : nullptr;
@@ -195,17 +178,13 @@ __device__ __forceinline__ void encode_plane(const float *__restrict__ atlas, co
 #pragma unroll
     for (int k = 0; k < kQuads; ++k) {
       if (b.at[k] < 0) continue;
-      uint32_t b0 = 0, b1 = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (!((b.live[k] >> i) & 1u)) continue;
-        const uint32_t q = lpo_code_mul(b.v[k][i], lo, delta, rd, L);
-        if (c < 3) {
-          b0 |= (q >> 8) << (8 * i);
-          b1 |= (q & 255u) << (8 * i);
-        } else {
-          b0 |= q << (8 * i);
-        }
+      uint32_t q[4];
+      lpo_codes4(b.v[k], b.live[k], lo, delta, rd, L, q);
+      // low bytes, and the high ones of a position channel
+      uint32_t b0 = q[0] | (q[1] << 8) | (q[2] << 16) | (q[3] << 24), b1 = 0;
+      if (c < 3) {
+        b1 = __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
+        b0 = __byte_perm(__byte_perm(q[0], q[1], 0x0051), __byte_perm(q[2], q[3], 0x0051), 0x5410);
       }
       if (vec) {
         *reinterpret_cast<uint32_t *>(p0 + b.at[k]) = b0;
