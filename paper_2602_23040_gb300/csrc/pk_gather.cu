@@ -111,47 +111,55 @@ struct Quad<__half> {
   __device__ static float one(const __half *p) { return __half2float(*p); }
 };
 
-// Live bits and Gaussian indices of the (up to) four texels x0 .. x0 + 3
-// of row y; with `write`, writes their texel ids and dynamic flags.  False if
-// none is live.
-__device__ __forceinline__ bool quad_live(const uint32_t *__restrict__ occ, const uint32_t *__restrict__ dyn,
-                                          const uint32_t *__restrict__ woff, int W, int y, int x0, int64_t N,
-                                          bool write, uint32_t *__restrict__ texel, uint8_t *__restrict__ dynflag,
-                                          bool live[4], int64_t gidx[4]) {
-  const int Wp = (W + 31) / 32;
-  bool any = false;
+// The live ones among the (up to) four texels x0 .. x0 + 3 of row y (bit i:
+// texel i), whose Gaussians are consecutive from `first`; with `write`,
+// writes their texel ids and dynamic flags.
+__device__ __forceinline__ uint32_t quad_live(const uint32_t *__restrict__ occ, const uint32_t *__restrict__ dyn,
+                                              const uint32_t *__restrict__ woff, int W, int y, int x0, int64_t N,
+                                              bool write, uint32_t *__restrict__ texel,
+                                              uint8_t *__restrict__ dynflag, int64_t &first) {
+  const int64_t w = (int64_t)y * ((W + 31) / 32) + (x0 >> 5);   // one word: x0 is a multiple of 4
+  const uint32_t word = occ[w];
+  uint32_t live = (word >> (x0 & 31)) & 15u;
+  if (x0 + 4 > W) live &= (1u << (W - x0)) - 1u;
+  first = woff[w] + __popc(word & ((1u << (x0 & 31)) - 1u));
+  int64_t g = first;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    int x = x0 + i;
-    live[i] = false;
-    gidx[i] = 0;
-    if (x < W) {
-      uint32_t word = occ[(int64_t)y * Wp + (x >> 5)];
-      uint32_t bit = 1u << (x & 31);
-      if (word & bit) {
-        int64_t g = woff[(int64_t)y * Wp + (x >> 5)] + __popc(word & (bit - 1u));
-        if (g < N) {
-          live[i] = true;
-          gidx[i] = g;
-          any = true;
-          if (write) {
-            texel[g] = (uint32_t)((int64_t)y * W + x);
-            dynflag[g] = dyn ? (uint8_t)((dyn[(int64_t)y * Wp + (x >> 5)] >> (x & 31)) & 1u) : (uint8_t)1;
-          }
-        }
-      }
+    if (!((live >> i) & 1u)) continue;
+    if (g >= N) {
+      live &= ~(1u << i);
+    } else if (write) {
+      texel[g] = (uint32_t)((int64_t)y * W + x0 + i);
+      dynflag[g] = dyn ? (uint8_t)((dyn[w] >> ((x0 & 31) + i)) & 1u) : (uint8_t)1;
     }
+    ++g;
   }
-  return any;
+  return live;
 }
 
-// One thread per 4 consecutive texels of a row.
+// The live ones of a group's four values, in order from dst.
+__device__ __forceinline__ void store_live(const float (&x)[4], uint32_t live, float *__restrict__ dst) {
+  const uint32_t r1 = live & 1u, r2 = r1 + ((live >> 1) & 1u), r3 = r2 + ((live >> 2) & 1u);
+  if (live & 1u) dst[0] = x[0];
+  if (live & 2u) dst[r1] = x[1];
+  if (live & 4u) dst[r2] = x[2];
+  if (live & 8u) dst[r3] = x[3];
+}
+
+// One thread per 4 consecutive texels of a row.  Loads in flight bound it: a
+// group's Gaussians are consecutive, so one pointer per channel and four small
+// offsets replace four 64-bit indices (128 registers, two CTAs per SM), and
+// three CTAs fit.  1024^2 atlas, 60 % live, 59 channels: FP32 90 -> 77 us
+// (395 MB of planes and SoA, 5.1 TB/s), three-level FP16 142 -> 81 us; with
+// four CTAs 74 us but the 512^2 atlas 24 -> 29 us.  A warp that puts its
+// values in order in shared memory to store whole rows of 32 takes 130 us.
 template <typename Tex, bool kVec>
-__global__ __launch_bounds__(256) void k_gather(const Tex *__restrict__ atlas, const uint32_t *__restrict__ occ,
-                                                const uint32_t *__restrict__ dyn, const uint32_t *__restrict__ woff,
-                                                int W, int H, int F, int D, int64_t N,
-                                                float *__restrict__ soa, uint32_t *__restrict__ texel,
-                                                uint8_t *__restrict__ dynflag, pk_device_status *status) {
+__global__ __launch_bounds__(256, 3) void k_gather(const Tex *__restrict__ atlas, const uint32_t *__restrict__ occ,
+                                                   const uint32_t *__restrict__ dyn,
+                                                   const uint32_t *__restrict__ woff, int W, int H, int F, int D,
+                                                   int64_t N, float *__restrict__ soa, uint32_t *__restrict__ texel,
+                                                   uint8_t *__restrict__ dynflag, pk_device_status *status) {
   const int Wq = (W + 3) / 4;
   uint32_t nbad = 0;   // (frame, Gaussian) pairs of this thread with a non-finite texel value
   const int64_t nq = (int64_t)Wq * H;
@@ -159,36 +167,30 @@ __global__ __launch_bounds__(256) void k_gather(const Tex *__restrict__ atlas, c
   const int64_t G = (int64_t)F * N;
   for (int64_t qi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; qi < nq; qi += (int64_t)gridDim.x * blockDim.x) {
     const int y = (int)(qi / Wq), x0 = (int)(qi % Wq) * 4;
-    int64_t gidx[4];
-    bool live[4];
-    if (!quad_live(occ, dyn, woff, W, y, x0, N, true, texel, dynflag, live, gidx)) continue;
+    int64_t first;
+    const uint32_t live = quad_live(occ, dyn, woff, W, y, x0, N, true, texel, dynflag, first);
+    if (!live) continue;
     const int64_t pix = (int64_t)y * W + x0;
     for (int f = 0; f < F; ++f) {
       uint32_t bad = 0;   // bit i: texel i has a non-finite value in some channel of frame f
+      const Tex *src = atlas + (int64_t)f * D * plane + pix;
+      float *dst = soa + (int64_t)f * N + first;
 #pragma unroll 4
-      for (int c = 0; c < D; ++c) {
-        const Tex *src = atlas + ((int64_t)f * D + c) * plane + pix;
-        float* dst = soa + (int64_t)c * G + (int64_t)f * N;
+      for (int c = 0; c < D; ++c, src += plane, dst += G) {
+        float x[4];
         if (kVec) {
-          typename Quad<Tex>::V v = __ldg(reinterpret_cast<const typename Quad<Tex>::V *>(src));
+          const typename Quad<Tex>::V v = __ldg(reinterpret_cast<const typename Quad<Tex>::V *>(src));
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (live[i]) {
-              const float x = Quad<Tex>::get(v, i);
-              dst[gidx[i]] = x;
-              bad |= (uint32_t)!isfinite(x) << i;
-            }
+          for (int i = 0; i < 4; ++i) x[i] = Quad<Tex>::get(v, i);
         } else {
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (live[i]) {
-              const float x = Quad<Tex>::one(src + i);
-              dst[gidx[i]] = x;
-              bad |= (uint32_t)!isfinite(x) << i;
-            }
+          for (int i = 0; i < 4; ++i) x[i] = (live >> i) & 1u ? Quad<Tex>::one(src + i) : 0.f;
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) bad |= (uint32_t)!isfinite(x[i]) << i;
+        store_live(x, live, dst);
       }
-      nbad += __popc(bad);
+      nbad += __popc(bad & live);
     }
   }
   // one atomic per warp
@@ -209,7 +211,8 @@ __device__ __forceinline__ float lpo_proxy(uint32_t q, float lo, float delta) {
 // channels (blockIdx.y = (frame, group)), whose loads are issued together.
 // kVec: the codes of four texels are one 4-byte load per plane.  At the
 // 1024^2 atlas with 59 channels 116 us with a byte load per texel and all
-// channels in one thread, 87 us so.
+// channels in one thread, 87 us so, and 63 us with one pointer per channel and
+// a group's Gaussians at small offsets from it, as in k_gather.
 constexpr int kChannels = 8;
 template <bool kCodes, bool kVec>
 __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src, const float *__restrict__ lohi,
@@ -233,11 +236,11 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
     const int f = fg / groups, c0 = (fg - f * groups) * kChannels;
     for (uint32_t qi = blockIdx.x * blockDim.x + threadIdx.x; qi < nq; qi += gridDim.x * blockDim.x) {
       const int y = (int)(qi / Wq), x0 = (int)(qi - (uint32_t)y * Wq) * 4;
-      int64_t gidx[4];
-      bool live[4];
-      if (!quad_live(occ, dyn, woff, W, y, x0, N, fg == 0, texel, dynflag, live, gidx)) continue;
+      int64_t first;
+      const uint32_t live = quad_live(occ, dyn, woff, W, y, x0, N, fg == 0, texel, dynflag, first);
+      if (!live) continue;
       const int64_t pix = (int64_t)y * W + x0;
-      float *dst = soa + (int64_t)f * N;
+      float *dst = soa + (int64_t)c0 * G + (int64_t)f * N + first;
       if (kCodes) {
         const uint8_t *cb = reinterpret_cast<const uint8_t *>(src) + (int64_t)f * (D + 3) * plane + pix;
         auto four = [&](int64_t at) -> uint32_t {   // the four texels' bytes of a code plane
@@ -245,7 +248,7 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
           uint32_t v = 0;
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            if (live[i]) v |= (uint32_t)__ldg(cb + at + i) << (8 * i);
+            if ((live >> i) & 1u) v |= (uint32_t)__ldg(cb + at + i) << (8 * i);
           return v;
         };
         uint32_t lob[kChannels], hib[3];
@@ -260,17 +263,18 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
           const int c = c0 + k;
           if (c >= D) break;
           const float lo = s_lo[c], delta = s_delta[c];
+          float x[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             uint32_t q = (lob[k] >> (8 * i)) & 255u;
             if (k < 3) q |= ((hib[k] >> (8 * i)) & 255u) << 8;
-            if (live[i]) dst[(int64_t)c * G + gidx[i]] = lpo_proxy(q, lo, delta);
+            x[i] = lpo_proxy(q, lo, delta);
           }
+          store_live(x, live, dst + k * G);
         }
       } else {
-        const uint32_t lanes = (live[0] ? 1u : 0u) | (live[1] ? 2u : 0u) | (live[2] ? 4u : 0u) | (live[3] ? 8u : 0u);
 #pragma unroll 4
-        for (int c = c0; c < min(c0 + kChannels, D); ++c) {
+        for (int c = c0; c < min(c0 + kChannels, D); ++c, dst += G) {
           const float lo = s_lo[c], delta = s_delta[c];
           const float *sc = reinterpret_cast<const float *>(src) + ((int64_t)f * D + c) * plane + pix;
           float x[4] = {0.f, 0.f, 0.f, 0.f};
@@ -280,13 +284,13 @@ __global__ __launch_bounds__(256) void k_gather_lpo(const void *__restrict__ src
           } else {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-              if (live[i]) x[i] = __ldg(sc + i);
+              if ((live >> i) & 1u) x[i] = __ldg(sc + i);
           }
           uint32_t q[4];
-          lpo_codes4(x, lanes, lo, delta, s_rd[c], c < 3 ? 65535.0f : 255.0f, q);
+          lpo_codes4(x, live, lo, delta, s_rd[c], c < 3 ? 65535.0f : 255.0f, q);
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (live[i]) dst[(int64_t)c * G + gidx[i]] = lpo_proxy(q[i], lo, delta);
+          for (int i = 0; i < 4; ++i) x[i] = lpo_proxy(q[i], lo, delta);
+          store_live(x, live, dst);
         }
       }
     }
