@@ -76,8 +76,8 @@ struct AdjSums {
 // splat, dL/do being -sum dq / o.  A pixel that skips the splat (ok false:
 // outside the footprint, or past its last blended entry) takes alpha 0,
 // which leaves its T and GS unchanged and adds 0 to every sum, so the pair
-// runs without a branch: its exponent is replaced, which makes 2^power and
-// all that follows from it 0 with no further select.  GS is kept negated
+// runs without a branch: its exponent is replaced, which makes 2^power, alpha
+// and the colour terms 0 with no further select (dq has one).  GS is kept negated
 // (NGS = -dL/dC . S) and alpha as nal = -alpha (the staged opacity is
 // negated), which turns dL/dalpha into one fused multiply-add.  kFirst: this
 // pair starts the sums instead of adding to them.
@@ -116,8 +116,12 @@ __device__ __forceinline__ void pixel_adjoint2(const float4 &a, const float4 &b,
   s.a6 = kFirst ? mul2(nwT, g0) : fma2(nwT, g0, s.a6);
   s.a7 = kFirst ? mul2(nwT, g1) : fma2(nwT, g1, s.a7);
   s.a8 = kFirst ? mul2(nwT, g2) : fma2(nwT, g2, s.a8);
-  // a clamped alpha does not depend on the exponent
-  const f32x2 dq = mul2(pack2(r0 < -kAlphaMax ? 0.f : r0, r1 < -kAlphaMax ? 0.f : r1), da);
+  // a clamped alpha does not depend on the exponent; selected after the
+  // product, so that a non-finite dL/dimage stays with the splats that blend
+  // there (0 times it would be NaN)
+  float dq0, dq1;
+  unpack2(mul2(pack2(r0, r1), da), dq0, dq1);
+  const f32x2 dq = pack2(ok0 && !(r0 < -kAlphaMax) ? dq0 : 0.f, ok1 && !(r1 < -kAlphaMax) ? dq1 : 0.f);
   const f32x2 t = mul2(dq, dy);
   s.q1 = kFirst ? dq : add2(s.q1, dq);
   s.qy = kFirst ? t : add2(s.qy, t);
