@@ -176,14 +176,6 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 2 ? 10 : 1)) void k_ras
               stage_from(s_raw[3 * j], s_raw[3 * j + 1], s_raw[3 * j + 2], s_pid[j], st, j);
             }
           }
-        if (may_hand && tid == 0) {
-          const uint32_t slot = few_left(rq, few) ? atomicAdd(&rq->items, 1u) : kNoPair;
-          if (slot < long_items) {
-            longs.w[slot] = w;
-            longs.first[slot] = walked;
-          }
-          s_hand[(walked >> 8) & 1u] = slot;
-        }
         fence_proxy_async();   // these reads of s_raw before the next bulk writes into it
         const uint64_t nxt = base + kBatch;
         const int nbn = nxt < e ? (int)min((uint64_t)kBatch, e - nxt) : 0;
@@ -191,6 +183,16 @@ __global__ __launch_bounds__(Geo<kPx>::kThreads, (kPx == 2 ? 10 : 1)) void k_ras
         if (__syncthreads_or(timed_out)) {
           timed_out = true;
           break;
+        }
+        // a slot only for a batch that arrived: one taken before the barrier
+        // above would go to the other kernel without its state
+        if (may_hand && tid == 0) {
+          const uint32_t slot = few_left(rq, few) ? atomicAdd(&rq->items, 1u) : kNoPair;
+          if (slot < long_items) {
+            longs.w[slot] = w;
+            longs.first[slot] = walked;
+          }
+          s_hand[(walked >> 8) & 1u] = slot;
         }
         if (nbn > 0) {
           fetch(nxt, nbn);
