@@ -1430,7 +1430,8 @@ int digit_base(bool entries, int blocks, int parts, uint64_t items) {
 // Block table of a segmented sort: per view a share of `nblocks`
 // proportional to weight(v) (at least one), each {view, part, parts, first
 // histogram counter}.  Returns the number of blocks, or 0 when the views do
-// not fit the histogram; *most = the largest number of parts.
+// not fit the histogram; *most = the largest number of parts.  tab: null to
+// count only.
 template <typename Weight>
 int share_blocks(int V, int nblocks, int cap, int rb, const Weight &weight, int4 *tab, int *most) {
   int64_t total = 0;
@@ -1440,7 +1441,7 @@ int share_blocks(int V, int nblocks, int cap, int rb, const Weight &weight, int4
   for (int v = 0; v < V; ++v) {
     const int parts = std::max<int>(1, (int)((int64_t)nblocks * weight(v) / std::max<int64_t>(1, total)));
     if (nb + parts > cap) return 0;
-    for (int j = 0; j < parts; ++j) tab[nb + j] = make_int4(v, j, parts, (1 << rb) * nb);
+    for (int j = 0; tab && j < parts; ++j) tab[nb + j] = make_int4(v, j, parts, (1 << rb) * nb);
     nb += parts;
     *most = std::max(*most, parts);
   }
@@ -1450,9 +1451,9 @@ int share_blocks(int V, int nblocks, int cap, int rb, const Weight &weight, int4
 }  // namespace
 
 // The tile passes' table (shares by tiles; tab[0, cap)) and the depth
-// passes' (equal shares: every view has N pairs at most; tab[cap, 2 cap));
-// `false` in the result's ntile: the plan sorts unsegmented (one view, or too
-// many views for the histogram).
+// passes' (equal shares: every view has N pairs at most; tab[cap, 2 cap)),
+// with tab null the numbers of blocks alone; seg false in the result: the
+// plan sorts unsegmented (one view, or too many views for the histogram).
 pk::SortBlocks pk::sort_layout(const pk_plan *p, int cap, int4 *tab) {
   const int rt = p->opts.sort_bits_tile, rd = p->opts.sort_bits_depth;
   const uint64_t pairs = (uint64_t)p->pairs, maxd = p->max_dups;
@@ -1464,7 +1465,7 @@ pk::SortBlocks pk::sort_layout(const pk_plan *p, int cap, int4 *tab) {
     const int nt = share_blocks(p->V, part_count(true, rt, maxd, kSegWaves, room), cap, rt,
                                 [&](int v) { return (int64_t)p->h_views[v].tiles_x * p->h_views[v].tiles_y; }, tab, &mt);
     const int np = share_blocks(p->V, part_count(false, rd, pairs, kSegWaves, room), cap, rd,
-                                [](int) { return int64_t(1); }, tab + cap, &mp);
+                                [](int) { return int64_t(1); }, tab ? tab + cap : nullptr, &mp);
     if (nt != 0 && np != 0) {
       b.seg = true;
       b.ntile = nt;
@@ -1525,8 +1526,8 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
   const int sms = sm_count();
   // segmented sorts (V >= 2): the depth passes sort each view's pairs in
   // place, the tile passes each view's entries on per-view local tile ids
-  int4 tab_host[2 * kSortBlocks];
-  const SortBlocks blk = sort_layout(p, L.sort_cap, tab_host);
+  // (the tables themselves were uploaded with the workspace)
+  const SortBlocks blk = sort_layout(p, L.sort_cap, nullptr);
   const bool seg = blk.seg;
   const int4 *tab = at<int4>(ws, L.sblk);
   uint64_t *vseg = at<uint64_t>(ws, L.vseg), *pseg = vseg + (p->V + 1);
@@ -1630,8 +1631,7 @@ pk_status bin_and_sort_impl(const pk_plan *p, const WsLayout &L, void *ws, const
 int pk::bin_kernel_count(const pk_plan *p) {
   if (!p) return 0;
   if (p->pairs == 0) return 1;
-  int4 tab[2 * kSortBlocks];
-  const SortBlocks blk = sort_layout(p, p->ws.sort_cap, tab);
+  const SortBlocks blk = sort_layout(p, p->ws.sort_cap, nullptr);
   int widths[8];
   auto launches = [](int base) { return base == kScan ? 4 : base == kDirect ? 2 : 1; };
   int kernels = 3 + 2 + 1 + 1;

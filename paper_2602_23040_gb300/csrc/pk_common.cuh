@@ -142,8 +142,8 @@ int resident_ctas(KernelInfo &info, const void *kernel, int threads, size_t smem
 pk_status zero_async(std::initializer_list<std::pair<void *, size_t>> spans, cudaStream_t st);
 // Radix blocks of the tile and depth passes on the current device, whether
 // they sort view by view (seg; then tab[0, cap) is the tile passes' block
-// table and tab[cap, 2 cap) the depth passes') and where their downsweeps take
-// the digit positions from (DigitBase, pk_binsort.cu).
+// table and tab[cap, 2 cap) the depth passes'; tab may be null) and where
+// their downsweeps take the digit positions from (DigitBase, pk_binsort.cu).
 struct SortBlocks {
   bool seg;
   int ntile, npair, tile_base, pair_base;
