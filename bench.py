@@ -207,12 +207,12 @@ def measured_fp32_per_eval(stage):
     return None
 
 
-def launches_per_step(plan, sms):
+def launches_per_step(plan):
     # gather 2, project 1, bin_and_sort (as the library counts it), fwd with the loss 2 (zeroing +
-    # compositing), bwd 2 (zeroing + adjoint), scatter 1; where there are at most 100 work items per
-    # resident CTA (10 per SM), the handed-over long lists too: fwd 1, bwd 2 (sums and segments)
+    # compositing), bwd 2 (zeroing + adjoint), scatter 1; for a plan of at most 152,000 work items (the
+    # library's kLongMostItems) the handed-over long lists too: fwd 1, bwd 2 (sums and segments)
     blocks = int(plan.n_tiles) * (plan.tile // 16) ** 2
-    handed = blocks <= 100 * 10 * sms
+    handed = blocks <= 152000
     return 2 + 1 + int(plan.sizes.bin_kernels) + 5 + (3 if handed else 0)
 
 
@@ -661,7 +661,7 @@ def main():
         "roofline": roof,
         "stages_ms": stage_ms,
         "counts": {"dups": dups, "evals_fwd": evals_fwd, "evals_bwd": evals_bwd, "valid_pairs": int(st["valid_pairs"])},
-        "gpu_launches": launches_per_step(plan, sms) * args.steps,
+        "gpu_launches": launches_per_step(plan) * args.steps,
         "clocks": clk,
     }
 

@@ -1408,14 +1408,14 @@ pk_status radix_pass(bool entries, int rb, const uint32_t *kin, const uint32_t *
 }
 
 // Blocks of an unsegmented pass over at most `items` pairs or entries, or
-// (waves > 1) the blocks that a segmented one shares out.
-int part_count(bool entries, int rb, uint64_t items, int waves, int cap) {
+// (waves > 1) the blocks that a segmented one shares out, on `sms` SMs.
+int part_count(bool entries, int rb, uint64_t items, int waves, int cap, int sms) {
   const int tile = kThreads * (entries ? kEntryItems : kPairItems);
   const int per_sm = entries ? (rb > 8 ? Radix<11, kEntryItems>::kMinBlocks : Radix<8, kEntryItems>::kMinBlocks)
                              : (rb > 8 ? Radix<11, kPairItems>::kMinBlocks : Radix<8, kPairItems>::kMinBlocks);
   if (waves == 1 && items <= (uint64_t)tile * kSoloTiles) return 1;
   const uint64_t useful = (items + (uint64_t)tile - 1) / (uint64_t)tile;
-  const uint64_t most = (uint64_t)std::min(cap, waves * per_sm * sm_count());
+  const uint64_t most = (uint64_t)std::min(cap, waves * per_sm * sms);
   return (int)std::max<uint64_t>(1, std::min(useful, most));
 }
 
@@ -1448,23 +1448,26 @@ int share_blocks(int V, int nblocks, int cap, int rb, const Weight &weight, int4
   return nb;
 }
 
+// Blocks to share out among V views: room for the one that a view takes at least.
+int seg_room(int V, int cap) { return std::max(1, cap - std::min(V, cap / 2)); }
+
 }  // namespace
 
 // The tile passes' table (shares by tiles; tab[0, cap)) and the depth
 // passes' (equal shares: every view has N pairs at most; tab[cap, 2 cap)),
 // with tab null the numbers of blocks alone; seg false in the result: the
-// plan sorts unsegmented (one view, or too many views for the histogram).
+// plan sorts unsegmented (one view, or too many views for `cap` blocks).
 pk::SortBlocks pk::sort_layout(const pk_plan *p, int cap, int4 *tab) {
   const int rt = p->opts.sort_bits_tile, rd = p->opts.sort_bits_depth;
   const uint64_t pairs = (uint64_t)p->pairs, maxd = p->max_dups;
+  const int sms = std::min(sm_count(), kSms);   // the plan holds counters for no more
   SortBlocks b{};
   if (p->V >= 2) {
-    // room for the one block a view takes at least
-    const int room = std::max(1, cap - std::min(p->V, cap / 2));
+    const int room = seg_room(p->V, cap);
     int mt = 0, mp = 0;
-    const int nt = share_blocks(p->V, part_count(true, rt, maxd, kSegWaves, room), cap, rt,
+    const int nt = share_blocks(p->V, part_count(true, rt, maxd, kSegWaves, room, sms), cap, rt,
                                 [&](int v) { return (int64_t)p->h_views[v].tiles_x * p->h_views[v].tiles_y; }, tab, &mt);
-    const int np = share_blocks(p->V, part_count(false, rd, pairs, kSegWaves, room), cap, rd,
+    const int np = share_blocks(p->V, part_count(false, rd, pairs, kSegWaves, room, sms), cap, rd,
                                 [](int) { return int64_t(1); }, tab ? tab + cap : nullptr, &mp);
     if (nt != 0 && np != 0) {
       b.seg = true;
@@ -1475,11 +1478,29 @@ pk::SortBlocks pk::sort_layout(const pk_plan *p, int cap, int4 *tab) {
       return b;
     }
   }
-  b.ntile = part_count(true, rt, maxd, 1, cap);
-  b.npair = part_count(false, rd, pairs, 1, cap);
+  b.ntile = part_count(true, rt, maxd, 1, cap, sms);
+  b.npair = part_count(false, rd, pairs, 1, cap, sms);
   b.tile_base = digit_base(true, b.ntile, b.ntile, maxd);
   b.pair_base = digit_base(false, b.npair, b.npair, pairs);
   return b;
+}
+
+// 8 bytes per digit and block, for the most blocks that sort_layout can give
+// (a segmented pass: those shared out and one more per view).  As many as the
+// keys fill, so 1 MB for a 64^2 atlas with one 256^2 view and 21 MB for the
+// 52-view rig; counters for kSortBlocks blocks of 11-bit digits took 42 MB in
+// every plan.
+size_t pk::sort_hist_bytes(const pk_plan *p, int cap) {
+  size_t most = 0;
+  for (const int rb : {8, kMaxRadixBits})
+    for (const bool entries : {false, true}) {
+      const uint64_t items = entries ? p->max_dups : (uint64_t)p->pairs;
+      int blocks = part_count(entries, rb, items, 1, cap, kSms);
+      if (p->V >= 2)
+        blocks = std::max(blocks, std::min(cap, part_count(entries, rb, items, kSegWaves, seg_room(p->V, cap), kSms) + p->V));
+      most = std::max(most, (sizeof(uint64_t) << rb) * (size_t)blocks);
+    }
+  return most;
 }
 
 namespace {

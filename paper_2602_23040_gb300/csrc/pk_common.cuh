@@ -29,16 +29,21 @@ constexpr float kDetMin = 1e-7f;
 constexpr float kExpScale = -0.72134752044448170f;
 constexpr float kInvExpScale = -1.38629436111989061f;   // 1 / kExpScale = -2 ln 2
 
+// SMs of the GB300: what a plan's buffers are sized for, whatever device it
+// is made on.
+constexpr int kSms = 152;
+
 // Fixed grid sizes of the device-count-driven kernels (scan, radix sort).
 constexpr int kScanBlocks = 4096;
-constexpr int kSortBlocks = 2560;     // most radix blocks of one pass (histogram capacity)
+constexpr int kSortBlocks = 2560;     // most radix blocks of one pass
 constexpr int kMaxRadixBits = 11;     // widest radix digit (pk_options.sort_bits_*: 8 or 11)
 constexpr uint64_t kMaxEntries = uint64_t(1) << 35;   // most (pair, tile) entries of a plan
 
-// Long lists (pk_raster.cuh): most of a pass, and most segments of the
+// Long lists (pk_raster.cuh): most of a pass -- one per CTA that is left when
+// the backward hands over, a quarter of 16 per SM -- and most segments of the
 // backward's in a pass.
-constexpr uint32_t kLongMaxItems = 1024;
-constexpr uint32_t kSplitMaxUnits = 24576;
+constexpr uint32_t kLongMaxItems = 4 * kSms;
+constexpr uint32_t kSplitMaxUnits = 128 * 64 + (kLongMaxItems - 128) * 16;   // (split_segments)
 constexpr uint32_t kSplitBlock = 256;   // pixels of a 16 x 16 block
 
 // Per-view constants on the device, 144 bytes.
@@ -88,7 +93,7 @@ struct WsLayout {
   size_t dkey0, dkey1, dval;
   size_t sblk, vseg;       // segmented sorts: block tables [2][sort_cap] int4 (tile passes, depth
                            // passes), view starts [2][V + 1] (entries, pairs)
-  int sort_cap;            // most radix blocks of one pass (counters in hist)
+  int sort_cap;            // most radix blocks of one pass
   size_t mask_tmp;         // one motion mask's worth of words (dilation scratch)
   size_t mask_coarse;      // per view, one bit per 32 x 32-pixel block: any moving pixel
   size_t longs, split;     // the forward's long lists and the backward's split lists (pk_raster.cuh)
@@ -107,7 +112,8 @@ struct pk_plan {
   int32_t tile_bits;       // bits needed for a global tile id
   int32_t num_sms;
   uint32_t first_polls;    // polls of the first bounded wait on a bulk-copied batch
-  uint32_t long_items, split_units;   // long lists (forward) and segments of split ones that the workspace holds
+  uint32_t long_items, split_units;   // long lists and segments of split ones that the workspace holds (0: the
+                                      // compositing walks every list whole)
   pk::WsLayout ws;
   pk::DevView *h_views;    // host copies uploaded by pk_workspace_init
   uint32_t *h_toff;        // [V+1] tile offsets (global tile id -> view)
@@ -149,6 +155,9 @@ struct SortBlocks {
   int ntile, npair, tile_base, pair_base;
 };
 SortBlocks sort_layout(const pk_plan *p, int cap, int4 *tab);
+// Bytes of digit counters that the plan's radix passes need on kSms SMs, with
+// digits of either width.
+size_t sort_hist_bytes(const pk_plan *p, int cap);
 // Kernels one pk_bin_and_sort call launches for this plan on this device.
 int bin_kernel_count(const pk_plan *p);
 

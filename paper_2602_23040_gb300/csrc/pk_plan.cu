@@ -346,7 +346,7 @@ extern "C" pk_status pk_plan_create(const pk_atlas_desc *desc, const pk_view *vi
   L.blocksums = take(sizeof(uint64_t) * (kScanBlocks + 1));
   // digit counters of the widest radix pass (room for 11-bit digits, so
   // that pk_autotune may pick them)
-  L.hist = take(sizeof(uint64_t) * (size_t(1) << kMaxRadixBits) * kSortBlocks);
+  L.hist = take(sort_hist_bytes(p, kSortBlocks));
   L.dkey0 = take(sizeof(uint32_t) * maxd);
   L.dkey1 = take(sizeof(uint32_t) * maxd);
   L.dval = take(sizeof(uint32_t) * maxd);
@@ -355,12 +355,14 @@ extern "C" pk_status pk_plan_create(const pk_atlas_desc *desc, const pk_view *vi
   L.vseg = take(sizeof(uint64_t) * 2 * (V + 1));
   L.mask_tmp = take(sizeof(uint32_t) * (size_t)p->mask_words);
   L.mask_coarse = take(sizeof(uint32_t) * (size_t)p->coarse_words);
-  // long lists (at most one per work item, and per CTA of the last few) and segments of
-  // split ones (64 entries at least, four quadrants' lists per tile)
-  const uint64_t blocks16 = (uint64_t)p->n_tiles * (o.tile / kTileSide) * (o.tile / kTileSide);
-  p->long_items = (uint32_t)std::min<uint64_t>(kLongMaxItems, blocks16);
+  // long lists (at most one per work item, and per CTA of the last few) and segments of split ones (64
+  // entries at least, a tile's list once per 16 x 16 quadrant), where the plan hands lists over: 37 MB at most
+  const uint64_t quads = (uint64_t)(o.tile / kTileSide) * (o.tile / kTileSide), blocks16 = (uint64_t)p->n_tiles * quads;
+  if (!o.count_evals && blocks16 <= (uint64_t)kLongMostItems) {
+    p->long_items = (uint32_t)std::min<uint64_t>(kLongMaxItems, blocks16);
+    p->split_units = (uint32_t)std::min<uint64_t>(kSplitMaxUnits, quads * maxd / 64 + 1);
+  }
   L.longs = take(LongItems::bytes(p->long_items));
-  p->split_units = (uint32_t)std::min<uint64_t>(kSplitMaxUnits, 4 * maxd / 64 + 1);
   L.split = take(SplitBwd::bytes(p->long_items, p->split_units));
   L.total = off;
   *out = p;

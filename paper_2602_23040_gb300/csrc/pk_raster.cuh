@@ -208,11 +208,13 @@ __device__ __forceinline__ bool block_may_hit(const float4 &box, const float4 &q
 // the instructions per entry, the backward's 1.4 times.  The lines lie at an eighth and a quarter of the resident CTAs:
 // with the hand-over as soon as the tile queue is dry instead, 44 views of
 // 195 x 195 pixels on 253 K splats take 11.1 ms for 6.7 (whole lists: 9.2).
-// And passes of more than kLongPasses work items per resident CTA run
-// without it: their tail is short, and the test in its loop costs the
-// forward 2 % (52-view rig, 306 K items: 4.11 -> 4.20 ms; at 66 K items a
-// 16-view step gains 13 %).
-constexpr int64_t kLongPasses = 100;
+// And passes of more than kLongMostItems work items (1,000 per SM, 100 for each
+// of the forward's resident CTAs at its usual batch) run without it: their
+// tail is short, and the test in its loop costs the forward 2 % (52-view rig,
+// 306 K items: 4.11 -> 4.20 ms; at 66 K items a 16-view step gains 13 %).  Nor
+// do passes that count their evaluations.  The plan settles it (long_items),
+// since its workspace holds the state.
+constexpr int64_t kLongMostItems = int64_t(1000) * kSms;
 __device__ __forceinline__ bool few_left(const RasterQueue *q, uint32_t few) {
   return gridDim.x - *reinterpret_cast<const volatile uint32_t *>(&q->exited) <= few;
 }

@@ -637,8 +637,7 @@ pk_status rasterize_bwd(const pk_plan *p, const float *records, const uint32_t *
                              {&status->evals_bwd, sizeof(uint64_t)}},
                             st);
   if (ze != PK_OK) return ze;
-  const int side = p->T == 32 ? 2 : 1;
-  const bool split = p->n_tiles * side * side <= kLongPasses * (int64_t)sm_count() * 10;   // the forward's rule
+  const bool split = p->long_items > 0;
 #define PK_BWD_T(B, M, C, S)                                                                                \
   return p->T == 32 ? launch_bwd<B, M, 32, C, S>(p, records, sorted_vals, tile_ranges, T_final, n_contrib,    \
                                                  dL_dimage, grad2d, ws, ctr, status, st)                      \

@@ -633,8 +633,7 @@ pk_status rasterize_fwd(const pk_plan *p, const float *records, const uint32_t *
                              {&ctr->loss_acc, target ? 2 * sizeof(double) + sizeof(float) : 0}},
                             st);
   if (ze != PK_OK) return ze;
-  const int side = p->T == 32 ? 2 : 1;
-  const bool hand = p->n_tiles * side * side <= kLongPasses * (int64_t)sm_count() * 10;   // 10 resident CTAs per SM
+  const bool hand = p->long_items > 0;
 #define PK_FWD_T(B, M, C, H)                                                                                     \
   return p->T == 32 ? launch_fwd<B, M, 32, C, H>(p, records, sorted_vals, tile_ranges, image, T_final, n_contrib, \
                                                  ws, ctr, status, target, dimg, clear, clear_floats, st)           \
