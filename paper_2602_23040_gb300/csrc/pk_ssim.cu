@@ -3,15 +3,15 @@
 //
 // One CTA per 32 x 32 output tile of one channel of one view.  It stages
 // the 52 x 52 input window of image and target (halo 2 x 5) in shared
-// memory, forms the four window sums (X, Y, XX + YY, XY: the SSIM
-// value needs the variances' sum alone) on the 42 x 42
-// region (halo 5) by a horizontal then a vertical 11-tap pass, turns them
-// into the SSIM value and its partial derivatives, and sums those back onto
-// the 32 x 32 tile with the same separable window (the adjoint of the
-// window sums).  Every pass is register-tiled: a thread produces 4 to 8
+// memory, forms the four window sums (X, Y, (X - Y)^2, XY: the SSIM value
+// needs the variances' sum alone, twice the covariance plus the variance of
+// X - Y) on the 42 x 42 region (halo 5) by a horizontal then a vertical
+// 11-tap pass, turns them into the SSIM value and its partial derivatives,
+// and sums those back onto the 32 x 32 tile with the same separable window
+// (the adjoint of the window sums).  Every pass is register-tiled: a thread produces 4 to 8
 // consecutive outputs of one row or column from one sliding read of the
 // inputs, so shared-memory reads are about 1/4 of the multiply-adds.  The
-// sums travel in pairs -- (X, Y), (XX + YY, XY) and, backwards, (d1, d11)
+// sums travel in pairs -- (X, Y), ((X - Y)^2, XY) and, backwards, (d1, d11)
 // -- so each tap is one packed FP32 multiply-add per pair (two
 // round-to-nearest results, each the scalar one), and backwards one scalar
 // for d12.
@@ -26,6 +26,13 @@
 // and issue slots each take 1.5 to 1.9 ms of the 4.20 ms at the 52-view rig
 // (234 M values); a fifth sum and four reciprocals per value instead of two
 // took 4.72 ms.
+// Where image and target agree, both factors of the SSIM value are 1 less
+// the difference's share, which is taken directly instead of as XX + YY less
+// twice XY: bit-equal images have an SSIM of exactly 1, and all that is left of
+// their gradient is the rounding of its last sum.  RMS error of the SSIM's
+// gradient, 512^2 pixels, XX + YY -> this: a smooth image against itself
+// 5.4e-5 -> 2.9e-5, against itself with noise of 1e-3 1.8e-4 -> 1.2e-4 (of 1.9),
+// two random ones 7.4e-7 -> 7.3e-7 (of 3.3).
 #include "pk_common.cuh"
 #include "pk_f32x2.cuh"
 
@@ -60,7 +67,7 @@ struct SsimSmem {
       float d2[kM][kMP];
     };
   };
-  f32x2 h01[kI][kMP], h23[kI][kMP];   // horizontal sums (X, Y), (XX + YY, XY); later the backward
+  f32x2 h01[kI][kMP], h23[kI][kMP];   // horizontal sums (X, Y), ((X - Y)^2, XY); later the backward
 };                                    //   sums (d1, d11) in h01 and d12 in h23, on [kM][kTP]
 static_assert(sizeof(float) * 2 * kM * kMP + sizeof(float) * kM * kMP <= sizeof(float) * 2 * kI * kIP,
               "the derivative maps fit in the input tiles they replace");
@@ -115,7 +122,7 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
     }
   }
   __syncthreads();
-  // B: horizontal window sums of X, Y, XX + YY, XY: each item one input row
+  // B: horizontal window sums of X, Y, (X - Y)^2, XY: each item one input row
   // and kGB consecutive window-sum columns (threads walk down the rows)
   for (int it = tid; it < kI * (kM / kGB); it += kSsimThreads) {
     const int g = it / kI, r = it - g * kI, q0 = g * kGB;
@@ -130,7 +137,8 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
       const f32x2 v = S.xy[r][q0 + t];
       float xv, yv;
       unpack2(v, xv, yv);
-      const f32x2 sq = pack2(fmaf(xv, xv, yv * yv), xv * yv);
+      const float dv = xv - yv;
+      const f32x2 sq = pack2(dv * dv, xv * yv);
 #pragma unroll
       for (int o = 0; o < kGB; ++o) {
         const int j = t - o;
@@ -149,7 +157,10 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
   // C: vertical window sums on kGC consecutive rows of one column, then the
   // SSIM value s = (A1 / B1) (A2 / B2) and its partial derivatives with
   // respect to m1 = G*X, e11 = G*XX, e12 = G*XY (0 outside the image); s's
-  // factors p = A1 / B1 and q = A2 / B2 leave two reciprocals per value
+  // factors p = A1 / B1 and q = A2 / B2 leave two reciprocals per value.  B1
+  // exceeds A1 by (m1 - m2)^2, B2 exceeds A2 by the variance of X - Y: the
+  // factors are 1 less u1 and u2, those over B1 and B2.  d1 and d12 are half
+  // of the derivatives; a value's gradient is 2 (G*d1 + X G*d11 + Y G*d12)
   float ssim_sum = 0.f;
   for (int it = tid; it < kM * (kM / kGC); it += kSsimThreads) {
     const int g = it / kM, q = it - g * kM, r0 = g * kGC;
@@ -176,18 +187,18 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
       const int r = r0 + o, yy = ty0 - kR + r;
       float d1 = 0.f, d11 = 0.f, d12 = 0.f;
       if (yy >= 0 && yy < H && xx >= 0 && xx < W) {
-        float m1, m2, ee, e12;
+        float m1, m2, edd, e12;
         unpack2(a01[o], m1, m2);
-        unpack2(a23[o], ee, e12);
-        const float m12 = m1 * m2, mm = fmaf(m1, m1, m2 * m2);
-        const float A1 = fmaf(2.f, m12, kC1), A2 = fmaf(2.f, e12 - m12, kC2);
-        const float B1 = mm + kC1, B2 = (ee - mm) + kC2;
+        unpack2(a23[o], edd, e12);
+        const float m12 = m1 * m2, dm = m1 - m2, dm2 = dm * dm, vd = edd - dm2;
+        const float B1 = fmaf(2.f, m12, kC1) + dm2, B2 = fmaf(2.f, e12 - m12, kC2) + vd;
         // approximate reciprocals (2 ulp): far inside the FP32 tolerance of the loss
         const float iB1 = __fdividef(1.f, B1), iB2 = __fdividef(1.f, B2);
-        const float p = A1 * iB1, qf = A2 * iB2, s = p * qf, pB2 = p * iB2;
-        d1 = 2.f * fmaf(m2, fmaf(qf, iB1, -pB2), m1 * (s * (iB2 - iB1)));
+        const float u1 = dm2 * iB1, u2 = vd * iB2;
+        const float p = 1.f - u1, qf = 1.f - u2, s = p * qf;
+        d12 = p * iB2;
         d11 = -s * iB2;
-        d12 = 2.f * pB2;
+        d1 = fmaf(iB1 * qf, fmaf(m1, u1, -dm), d12 * fmaf(-m1, u2, dm));
         if (r >= kR && r < kR + kT && q >= kR && q < kR + kT) ssim_sum += s;
       }
       S.d01[r][q] = pack2(d1, d11);
@@ -231,7 +242,7 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
   // (read again from global memory: their shared copy now holds the
   // derivative maps) and the L1 term
   float l1_sum = 0.f;
-  const float gl1 = (1.f - lambda) * inv_n, gs = lambda * inv_n;
+  const float gl1 = (1.f - lambda) * inv_n, gs = 2.f * lambda * inv_n;
   for (int it = tid; it < kT * (kT / kGE); it += kSsimThreads) {
     const int g = it / kT, q = it - g * kT, r0 = g * kGE;
     const int xx = tx0 + q;
@@ -262,11 +273,11 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
       const float xv = __ldg(X + (int64_t)yy * W + xx), yv = __ldg(Y + (int64_t)yy * W + xx);
       float s0, s1;
       unpack2(c01[o], s0, s1);
-      const float dS = s0 + 2.f * xv * s1 + yv * c2[o];
+      const float hS = fmaf(yv, c2[o], fmaf(xv, s1, s0));   // half the SSIM's gradient
       const float dd = xv - yv;
       l1_sum += fabsf(dd);
       const float sg = dd > 0.f ? 1.f : (dd < 0.f ? -1.f : 0.f);
-      grad[3 * view.pix_off + c * plane + (int64_t)yy * W + xx] = gl1 * sg - gs * dS;
+      grad[3 * view.pix_off + c * plane + (int64_t)yy * W + xx] = gl1 * sg - gs * hS;
     }
   }
   // block sums of L1 and SSIM, one double atomic each
