@@ -988,9 +988,10 @@ __global__ __launch_bounds__(kThreads, (Radix<RB, IT>::kMinBlocks)) void k_radix
     parity[cur] ^= 1u;
     uint32_t key[C::kItems], rank[C::kItems];
     // a tile whose keys all share one digit keeps its order: its run goes
-    // out as it is (tried only where that is likely -- the top byte of the
-    // depths, which all lie within a binade or two -- since the check costs
-    // a pass over the tile)
+    // out as it is (tried only in the last depth pass, since the check costs
+    // a pass over the tile: that pass runs only where the depths span 2^24
+    // floats or more, and where few outliers do that, most tiles hold its
+    // digit 0 alone)
     if (!kLast && try_single) {
       const uint32_t d0 = (bk[0] >> shift) & mask;   // valid >= 1 here
       bool same = true;
@@ -1388,8 +1389,7 @@ pk_status radix_pass(bool entries, int rb, const uint32_t *kin, const uint32_t *
                      const DevCounters *depth = nullptr, Unpack up = Unpack{}) {
 #define PK_PASS(RB, IT, M)                                                                                        \
   return radix_pass_rb<RB, IT, M>(kin, vin, kout, vout, n_dev, n_host, shift, bits, hist, nblocks, dbase, csum,   \
-                                  status,                                                                   \
-                                  sp, abort_flag, first_polls, try_single, depth, up, st)
+                                  status, sp, abort_flag, first_polls, try_single, depth, up, st)
   if (entries) {
     if (!vin && up.ranges) {
       if (rb > 8) PK_PASS(11, kEntryItems, 2);

@@ -24,9 +24,10 @@ __device__ __forceinline__ float lpo_rstep(float delta) {
 // value, the product lies within 2^-23 relative of the quotient and the sum
 // within 2 x 2^-24, so a sum u further than 1e-6 (1 + u) from an integer
 // has the quotient form's floor (below 0 either form's code is 0).  The
-// division for the others (position channels 2 lanes in 100, the rest 3 in
-// 10,000).  The four run without a branch per value, and one test leaves to
-// the division.
+// division for the others: 2e-6 (1 + u) of the values at a code u, so 3 in
+// 10,000 of the 8-bit channels' and, of the positions', 6.5 in 100 in the
+// middle of their range -- some lane of nearly every warp.  The four run
+// without a branch per value, and one test leaves to the division.
 __device__ __forceinline__ void lpo_codes4(const float (&x)[4], uint32_t live, float lo, float delta, float rd,
                                            float L, uint32_t (&q)[4]) {
   uint32_t unsure = 0;

@@ -48,7 +48,8 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // a word; any other view takes one pixel per lane, a ballot per word.
 // limit: the largest float whose (round-to-nearest) square root is <= tau, so
 // that |F| > tau is fx^2 + fy^2 > limit without the root.  225 -> 89 us at the
-// 52-view rig (77.9 M pixels, 7.0 TB/s).
+// 52-view rig (77.9 M pixels: 623 MB at 7.0 TB/s, reads alone and some of them
+// L2 hits, where a copy reaches 6.8).
 constexpr int kWordsPerWarp = 16;
 __global__ __launch_bounds__(kMaskThreads) void k_motion_threshold(const float *__restrict__ flow,
                                                                     const DevView *__restrict__ views, float limit,
@@ -301,10 +302,11 @@ __device__ __forceinline__ bool block_moves(const uint32_t *__restrict__ vcoarse
 // error near 2^-22 is far below the widening, so they too only ever skip
 // what cannot pass.  At the 52-view rig 607 -> 549 us with the square tested
 // first and, in the scan, the mask's words before the ellipse's rows, and
-// 534 us with the pixel at the mean.  The pairs whose rectangle reaches a moving block are then scanned one after
-// the other by the whole warp (warp_pair_hits), so that a long scan near
-// the motion does not run on one lane while the others wait.  A Gaussian
-// is marked at its first hit and takes no further views.
+// 534 us with the pixel at the mean.  The pairs whose rectangle reaches a
+// moving block are then scanned one after the other by the whole warp
+// (warp_pair_hits), so that a long scan near the motion does not run on one
+// lane while the others wait.  A Gaussian is marked at its first hit and takes
+// no further views.
 __global__ __launch_bounds__(kMaskThreads) void k_dynamic_mask(const float *__restrict__ rec,
                                                                 const uint32_t *__restrict__ texel,
                                                                 const uint32_t *__restrict__ mask,

@@ -57,9 +57,6 @@ __global__ void k_status_out(const uint32_t *__restrict__ st, int nst, const uin
 
 }  // namespace
 
-// One kernel instead of cudaMemsetAsync: inside a CUDA graph a memset node
-// may be run by a copy engine, where it queues behind (and is delayed by)
-// unrelated host <-> device copies of other streams.
 int sm_count() {
   static std::atomic<int> cached[64];
   int dev = 0;
@@ -84,6 +81,9 @@ int resident_ctas(KernelInfo &info, const void *kernel, int threads, size_t smem
   return n;
 }
 
+// One kernel instead of cudaMemsetAsync: inside a CUDA graph a memset node
+// may be run by a copy engine, where it queues behind (and is delayed by)
+// unrelated host <-> device copies of other streams.
 pk_status zero_async(std::initializer_list<std::pair<void *, size_t>> spans, cudaStream_t st) {
   ZeroSpans z{};
   uint64_t most = 0;

@@ -205,9 +205,10 @@ __device__ __forceinline__ bool block_may_hit(const float4 &box, const float4 &q
 // that spread one list over more of the GPU (k_raster_fwd_long, the backward's
 // segments below).  While more of them run, lists are walked whole, which
 // takes less work in all: the forward's other kernel spends about 2.4 times
-// the instructions per entry, the backward's 1.4 times.  The lines lie at an eighth and a quarter of the resident CTAs:
-// with the hand-over as soon as the tile queue is dry instead, 44 views of
-// 195 x 195 pixels on 253 K splats take 11.1 ms for 6.7 (whole lists: 9.2).
+// the instructions per entry, the backward's 1.4 times.  The lines lie at an
+// eighth (forward) and a quarter (backward) of the resident CTAs: with the
+// hand-over as soon as the tile queue is dry instead, 44 views of 195 x 195
+// pixels on 253 K splats take 11.1 ms for 6.7 (whole lists: 9.2).
 // And passes of more than kLongMostItems work items (1,000 per SM, 100 for each
 // of the forward's resident CTAs at its usual batch) run without it: their
 // tail is short, and the test in its loop costs the forward 2 % (52-view rig,
