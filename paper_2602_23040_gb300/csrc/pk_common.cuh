@@ -112,8 +112,8 @@ struct pk_plan {
   int32_t tile_bits;       // bits needed for a global tile id
   int32_t num_sms;
   uint32_t first_polls;    // polls of the first bounded wait on a bulk-copied batch
-  uint32_t long_items, split_units;   // long lists and segments of split ones that the workspace holds (0: the
-                                      // compositing walks every list whole)
+  uint32_t long_items, split_units;   // long lists and segments of split ones that the workspace holds (0: no list
+                                      // is handed over)
   pk::WsLayout ws;
   pk::DevView *h_views;    // host copies uploaded by pk_workspace_init
   uint32_t *h_toff;        // [V+1] tile offsets (global tile id -> view)

@@ -356,9 +356,10 @@ extern "C" pk_status pk_plan_create(const pk_atlas_desc *desc, const pk_view *vi
   L.mask_tmp = take(sizeof(uint32_t) * (size_t)p->mask_words);
   L.mask_coarse = take(sizeof(uint32_t) * (size_t)p->coarse_words);
   // long lists (at most one per work item, and per CTA of the last few) and segments of split ones (64
-  // entries at least, a tile's list once per 16 x 16 quadrant), where the plan hands lists over: 37 MB at most
+  // entries at least, a tile's list once per 16 x 16 quadrant), where the plan hands lists over: 37 MB at most.
+  // (Not less for a plan that counts its evaluations and so does not: its workspace serves the same plan without.)
   const uint64_t quads = (uint64_t)(o.tile / kTileSide) * (o.tile / kTileSide), blocks16 = (uint64_t)p->n_tiles * quads;
-  if (!o.count_evals && blocks16 <= (uint64_t)kLongMostItems) {
+  if (blocks16 <= (uint64_t)kLongMostItems) {
     p->long_items = (uint32_t)std::min<uint64_t>(kLongMaxItems, blocks16);
     p->split_units = (uint32_t)std::min<uint64_t>(kSplitMaxUnits, quads * maxd / 64 + 1);
   }

@@ -41,18 +41,18 @@ LIST, SEGMENT, MOST, MOST_SEGMENTS = 256 * 28 + 28, 256 * 8, 608, 128 * 64 + 480
     (1024, 0.6, [(1920, 1080)], 2 * 152, True),
     (1024, 0.6, RIG, 4 * 2 * 152 + 52, False)])                # four waves, one more per view; 306 K work items
 def test_workspace_beside_the_arrays(api, side, occ, sizes, blocks, hands):
-    whole = _beside_arrays(api, side, occ, sizes, count_evals=True)   # walks every list whole
-    assert whole <= blocks * COUNTERS + FIXED
     items = sum(math.ceil(w / 32) * math.ceil(h / 32) for w, h in sizes) * 4
-    lists = _beside_arrays(api, side, occ, sizes) - whole
-    if hands:
-        assert 0 < lists <= min(items, MOST) * LIST + MOST_SEGMENTS * SEGMENT + 1024
-    else:
-        assert lists == 0
+    lists = min(items, MOST) * LIST + MOST_SEGMENTS * SEGMENT if hands else 0
+    assert _beside_arrays(api, side, occ, sizes) <= blocks * COUNTERS + lists + FIXED
 
 
 def test_segments_follow_the_entries(api):
-    # 4 quadrants x 1,024 entries / 64 + 1 segments
-    lists = _beside_arrays(api, 16, 0.1, [(640, 480)], max_dups=1024) - \
-        _beside_arrays(api, 16, 0.1, [(640, 480)], max_dups=1024, count_evals=True)
-    assert lists <= MOST * LIST + 65 * SEGMENT + 1024
+    # 4 quadrants x 1,024 entries / 64 + 1 segments; one block's counters
+    beside = _beside_arrays(api, 16, 0.1, [(640, 480)], max_dups=1024)
+    assert beside <= COUNTERS + MOST * LIST + 65 * SEGMENT + FIXED
+
+
+def test_counting_plan_shares_the_workspace(api):
+    for sizes in ([(640, 480)], RIG):
+        a, b = (_beside_arrays(api, 64, 1.0, sizes, count_evals=c) for c in (False, True))
+        assert a == b
