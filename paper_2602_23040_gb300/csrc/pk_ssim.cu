@@ -23,16 +23,18 @@
 // stage reads its centre values again from global memory, where they are
 // still cached), which brings a CTA to 58 KB and three CTAs onto an SM.
 // Shared-memory wavefronts (about 75 per 32 values), packed multiply-adds
-// and issue slots each take 1.5 to 1.9 ms of the 4.20 ms at the 52-view rig
+// and issue slots each take 1.5 to 1.9 ms of the 4.23 ms at the 52-view rig
 // (234 M values); a fifth sum and four reciprocals per value instead of two
 // took 4.72 ms.
-// Where image and target agree, both factors of the SSIM value are 1 less
-// the difference's share, which is taken directly instead of as XX + YY less
-// twice XY: bit-equal images have an SSIM of exactly 1, and all that is left of
-// their gradient is the rounding of its last sum.  RMS error of the SSIM's
+// Where image and target agree, the SSIM's numerators and denominators differ
+// by the difference's variance and squared mean alone, taken directly instead
+// of as XX + YY less twice XY: bit-equal images have an SSIM of exactly 1, and
+// all that is left of their gradient is the rounding of its last sum.  RMS error of the SSIM's
 // gradient, 512^2 pixels, XX + YY -> this: a smooth image against itself
 // 5.4e-5 -> 2.9e-5, against itself with noise of 1e-3 1.8e-4 -> 1.2e-4 (of 1.9),
-// two random ones 7.4e-7 -> 7.3e-7 (of 3.3).
+// two random ones 7.4e-7 -> 7.3e-7 (of 3.3); a black image against a random
+// one 6.0e-9 (of 0.047), where 1 less the difference's share as the factors
+// left 1.9e-7.
 #include "pk_common.cuh"
 #include "pk_f32x2.cuh"
 
@@ -158,9 +160,9 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
   // SSIM value s = (A1 / B1) (A2 / B2) and its partial derivatives with
   // respect to m1 = G*X, e11 = G*XX, e12 = G*XY (0 outside the image); s's
   // factors p = A1 / B1 and q = A2 / B2 leave two reciprocals per value.  B1
-  // exceeds A1 by (m1 - m2)^2, B2 exceeds A2 by the variance of X - Y: the
-  // factors are 1 less u1 and u2, those over B1 and B2.  d1 and d12 are half
-  // of the derivatives; a value's gradient is 2 (G*d1 + X G*d11 + Y G*d12)
+  // exceeds A1 by (m1 - m2)^2, B2 exceeds A2 by the variance of X - Y.  d1 and
+  // d12 are half of the derivatives; a value's gradient is
+  // 2 (G*d1 + X G*d11 + Y G*d12)
   float ssim_sum = 0.f;
   for (int it = tid; it < kM * (kM / kGC); it += kSsimThreads) {
     const int g = it / kM, q = it - g * kM, r0 = g * kGC;
@@ -191,14 +193,17 @@ __global__ __launch_bounds__(kSsimThreads, 3) void k_photo(const float *__restri
         unpack2(a01[o], m1, m2);
         unpack2(a23[o], edd, e12);
         const float m12 = m1 * m2, dm = m1 - m2, dm2 = dm * dm, vd = edd - dm2;
-        const float B1 = fmaf(2.f, m12, kC1) + dm2, B2 = fmaf(2.f, e12 - m12, kC2) + vd;
-        // approximate reciprocals (2 ulp): far inside the FP32 tolerance of the loss
+        const float A1 = fmaf(2.f, m12, kC1), A2 = fmaf(2.f, e12 - m12, kC2);
+        const float B1 = A1 + dm2, B2 = A2 + vd;
+        // approximate reciprocals (2 ulp), the factors corrected by their
+        // remainders: exactly 1 where A = B, and right to the last bit or two
+        // however small
         const float iB1 = __fdividef(1.f, B1), iB2 = __fdividef(1.f, B2);
-        const float u1 = dm2 * iB1, u2 = vd * iB2;
-        const float p = 1.f - u1, qf = 1.f - u2, s = p * qf;
+        const float p0 = A1 * iB1, q0 = A2 * iB2;
+        const float p = fmaf(fmaf(-p0, B1, A1), iB1, p0), qf = fmaf(fmaf(-q0, B2, A2), iB2, q0), s = p * qf;
         d12 = p * iB2;
         d11 = -s * iB2;
-        d1 = fmaf(iB1 * qf, fmaf(m1, u1, -dm), d12 * fmaf(-m1, u2, dm));
+        d1 = fmaf(iB1 * qf, fmaf(-m1, p, m2), d12 * fmaf(m1, qf, -m2));
         if (r >= kR && r < kR + kT && q >= kR && q < kR + kT) ssim_sum += s;
       }
       S.d01[r][q] = pack2(d1, d11);
