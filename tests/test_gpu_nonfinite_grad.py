@@ -10,7 +10,7 @@ from tests import helpers as H
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-PX, PY = 10, 12   # the pixel, in the first 16 x 8 block's second row of blocks
+PX, PY = 10, 12   # in the left half of the tile: its warp holds a 16 x 8 block
 
 
 def _records(n, side):
